@@ -93,7 +93,7 @@ void free_dft2(tcu_dft2_plan_s *p) {
 
 // Column-pass TMA map: [array][row a][column v], GG columns x n1 rows.
 bool cols_map(CUtensorMap *m, const void *in, const tcu_dft2_plan_s *p) {
-  const long long gg = (128ll * p->r) / p->n1;
+  const long long gg = (128ll * p->cols.tw * p->r) / p->n1;
   return encode_map(m, in, p->n2, p->n1, p->batch, p->n1 * p->n2, (int)gg,
                     p->n1 < 256 ? (int)p->n1 : 256);
 }
@@ -242,8 +242,8 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   c.log2L = log2r * k1;
   c.U = batch * n2;
   c.modes[0] = c.modes[1] = c.modes[2] = kUF;
-  c.tw = 1;
-  c.swz_tab = choose_swizzle(r, c.s, c.modes, 1);
+  c.tw = team_size(r, c);
+  c.swz_tab = choose_swizzle(r, c.s, c.modes, c.tw);
   w.s = k2;
   w.role = kSingle;
   w.so = w.sp = w.lo = w.lp = 0;
@@ -252,8 +252,8 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   w.modes[0] = kQF;
   w.modes[1] = kUF;
   w.modes[2] = kRQF;
-  w.tw = 1;
-  w.swz_tab = choose_swizzle(r, w.s, w.modes, 1);
+  w.tw = team_size(r, w);
+  w.swz_tab = choose_swizzle(r, w.s, w.modes, w.tw);
   std::vector<float> conv_img;
   for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
     const int sign = d == 0 ? -1 : 1;

@@ -63,7 +63,14 @@ enum Role { kSingle = 0, kFirst = 1, kSecond = 2, kCols = 3, kSecondQ = 4 };
 
 __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 16 ? 4 : 5); }
 // Warpgroups per CTA: TMEM holds 512 columns, a warpgroup's slot 3 Q of
-// them; a radix-16 first (strided) pass also stages its inter-pass twiddles
+// them (Q = 2 R).  Radix 8 runs eight (slots of 48 columns, 64 registers a
+// thread): a row is only 8 values, so its threads are light and the pass is
+// bound by how many items are in flight (8^5 x 4096, five or four -> eight:
+// strided pass 362 -> 335 us, 3-stage team pass 515 -> 451 us; 8^4 x 16384
+// last pass 175 -> 167 us); the 3-stage radix-8 passes on one-warpgroup items,
+// which work mostly in shared memory, keep five (8^3 x 100000: 168 us against
+// 174).  A
+// radix-16 first (strided) pass also stages its inter-pass twiddles
 // in SMEM, which leaves room for four; a radix-16 last pass of several runs
 // four too (measured faster than five: 0.165 instead of 0.181 ms for the
 // second pass of n = 16^4 x 1024).  A radix-32 pass of two stages runs
@@ -72,11 +79,16 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // the convolution row pass and the fused schedule keep whole-K slots, two
 // per CTA at radix 32 (whole_k_nwg).
 __host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
-  return R == 32 ? (S >= 2 ? 4 : 2) : ((ROLE == 1 || ROLE == 2) && R == 16 ? 4 : 5);
+  return R == 8    ? (S == 3 ? 5 : 8)
+         : R == 32 ? (S >= 2 ? 4 : 2)
+                   : ((ROLE == 1 || ROLE == 2) && R == 16 ? 4 : 5);
 }
-__host__ __device__ constexpr int whole_k_nwg(int R, int ROLE) {
-  return R == 32 ? 2 : pass_nwg(R, ROLE);
+__host__ __device__ constexpr int whole_k_nwg(int R, int ROLE, int S = 2) {
+  return R == 32 ? 2 : pass_nwg(R, ROLE, S);
 }
+// Warpgroups per CTA of a team pass: two teams of four at radix 8, two teams
+// of two at radix 16 (TMEM: 96 columns a slot; SMEM).
+__host__ __device__ constexpr int team_nwg(int R) { return R == 8 ? 8 : 4; }
 
 // Compile-time geometry of one pass: S stages of radix R.  A transform of
 // length n is computed in up to three passes (the four-step split applied
@@ -142,7 +154,7 @@ struct Geo {
   static constexpr bool TW2L = TW_OUT && LOG2UPER > 8;
   static constexpr int TWB = (TW2L && TW_SMEM) ? L : 0;  // SMEM row of table B
   static constexpr int TMA_ROWS = L < 256 ? L : 256;  // tensor box height
-  static constexpr int Q = (2 * R > 32) ? 2 * R : 32;
+  static constexpr int Q = 2 * R;
   // half-K products (radix 32, four warpgroups): A regions of Q/2 columns
   static constexpr bool KS = R == 32 && NWG == 4 && TW == 1;
   static constexpr int QA = KS ? Q / 2 : Q;
@@ -405,7 +417,7 @@ __device__ __forceinline__ void split_store8(const float2 *x, uint32_t col_hi,
 //
 // HALF >= 0: only the products of K half HALF, with A (QA columns per
 // operand) holding that half; half 1 accumulates onto half 0.
-template <int R, int PREC, int QA = ((2 * R > 32) ? 2 * R : 32), int HALF = -1>
+template <int R, int PREC, int QA = 2 * R, int HALF = -1>
 __device__ __forceinline__ void issue_stage_mma(uint32_t slot, uint32_t img_addr) {
   constexpr bool BF = is_bf16(PREC);
   constexpr int IMG = img_bytes(R, PREC), LBO = 128, SBO = (BF ? 32 : 64) * R;
@@ -1207,11 +1219,11 @@ struct StaticNext {
 template <int R, int PREC, int S, int LO, int ROLE, int LP, bool CONV = false, int TW = 1>
 __global__ void __launch_bounds__(
     Geo<R, S, LO, ROLE, LP,
-        TW == 1 ? (CONV ? whole_k_nwg(R, ROLE) : pass_nwg(R, ROLE, S)) : 4, TW>::THREADS,
+        TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>::THREADS,
     1) dft_pass_kernel(const __grid_constant__ GArgs a) {
   using G =
-      Geo<R, S, LO, ROLE, LP, TW == 1 ? (CONV ? whole_k_nwg(R, ROLE) : pass_nwg(R, ROLE, S)) : 4,
-          TW>;
+      Geo<R, S, LO, ROLE, LP,
+          TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>;
   static_assert(!CONV || ROLE == kSingle, "convolution rows are whole transforms");
   using SM = SmemLayout<R, G::NWG, G::TW_ENTRIES, CONV ? G::TW_ENTRIES : 0, G::TW_SMEM, G::TWB,
                         TW, G::KS>;

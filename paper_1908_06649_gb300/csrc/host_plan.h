@@ -191,17 +191,15 @@ int plan_stages(int r, int k, int st[kMaxPasses]);
 // q, k = 1..3 for r = 8, k = 1..2 for r = 16 and 32.  Returns the number of
 // passes (0: not such an n) and fills the passes.
 int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]);
-// Warpgroups per item of pass pp: 4 for the 3-stage radix-8 passes of
-// two-pass transforms (an item of 512 rows holds 8 sub-transforms of 512
-// points, so the strided side moves 64-byte runs), else 1.
-int team_size(int r, int npasses, const PassPlan &pp);
+// Warpgroups per item of pass pp (its role and stages are set).
+int team_size(int r, const PassPlan &pp);
 // Role, neighbouring stage counts, size and row maps of pass `pi`.
 void pass_geometry(PassPlan &pp, int pi, int P, const int st[kMaxPasses], int k, int r,
                    long long n, long long batch);
 void free_plan(tcu_dft_plan_s *p);
 // ---------------------------------------------------------------- launches
 cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, int num_sms,
-                          cudaStream_t st, bool team_plan = false);
+                          cudaStream_t st);
 cudaError_t fused_dispatch(int r, int prec, int s1, int s2, const GArgs &a, int num_sms,
                            cudaStream_t st);
 // Warpgroup-kernel description of pass `pi` between buffers `in` and `out`.

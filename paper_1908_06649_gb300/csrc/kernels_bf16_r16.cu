@@ -4,7 +4,7 @@
 
 namespace tcu {
 
-cudaError_t launch_pass_bf16_r16(int prec, int s, int lo, int role, int lp, int tw,
+cudaError_t launch_pass_bf16_r16(int prec, int s, int lo, int role, int lp,
                                  const GArgs &a, int num_sms, cudaStream_t st) {
   constexpr int R = 16;
   TCU_BF16_TEAM_CASE(3, 0, kSingle, 0, 2)  // 16^3 in one pass

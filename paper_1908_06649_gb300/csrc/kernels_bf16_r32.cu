@@ -5,7 +5,7 @@
 
 namespace tcu {
 
-cudaError_t launch_pass_bf16_r32(int prec, int s, int lo, int role, int lp, int tw,
+cudaError_t launch_pass_bf16_r32(int prec, int s, int lo, int role, int lp,
                                  const GArgs &a, int num_sms, cudaStream_t st) {
   constexpr int R = 32;
   TCU_BF16_CASE(1, 0, kSingle, 0)

@@ -24,11 +24,12 @@ cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// A team pass: items of TW warpgroups (128 TW rows), four warpgroups a CTA.
+// A team pass: items of TW warpgroups (128 TW rows), team_nwg(R) warpgroups
+// a CTA.
 template <int R, int PREC, int S, int LO, int ROLE, int LP, int TW>
 cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
-  using G = Geo<R, S, LO, ROLE, LP, 4, TW>;
-  const size_t sm = SmemLayout<R, 4, G::TW_ENTRIES, 0, G::TW_SMEM, G::TWB, TW>::BYTES;
+  using G = Geo<R, S, LO, ROLE, LP, team_nwg(R), TW>;
+  const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, 0, G::TW_SMEM, G::TWB, TW>::BYTES;
   cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, false, TW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
@@ -40,18 +41,17 @@ cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-#define TCU_TEAM_CASE(S, SO, ROLE, SP, TW)                                               \
-  if (s == S && lo == log2_radix(R) * (SO) && role == ROLE && lp == log2_radix(R) * (SP) && \
-      tw == TW)                                                                           \
-    return prec == 3 ? launch_team_t<R, 3, S, log2_radix(R) * (SO), ROLE,               \
-                                     log2_radix(R) * (SP), TW>(a, num_sms, st)           \
-                     : launch_team_t<R, 1, S, log2_radix(R) * (SO), ROLE,               \
-                                     log2_radix(R) * (SP), TW>(a, num_sms, st);
+#define TCU_TEAM_CASE_L(S, LO, ROLE, LP, TW)                                             \
+  if (s == S && lo == LO && role == ROLE && lp == LP)                                     \
+    return prec == 3 ? launch_team_t<R, 3, S, LO, ROLE, LP, TW>(a, num_sms, st)           \
+                     : launch_team_t<R, 1, S, LO, ROLE, LP, TW>(a, num_sms, st);
+#define TCU_TEAM_CASE(S, SO, ROLE, SP, TW) \
+  TCU_TEAM_CASE_L(S, log2_radix(R) * (SO), ROLE, log2_radix(R) * (SP), TW)
 
 // The convolution row pass (forward rows, spectrum product, inverse rows).
 template <int R, int PREC, int S>
 cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
-  using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, kSingle)>;
+  using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, kSingle, S)>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::TW_ENTRIES, false, 0>::BYTES;
   cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, true>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -128,14 +128,14 @@ cudaError_t launch_pair_t(const GArgs &a, int clusters, cudaStream_t st) {
 // pass or a team pass (items of TW warpgroups).
 #define TCU_BF16_CASE(S, SO, ROLE, SP)                                                  \
   if (s == S && lo == log2_radix(R) * (SO) && role == ROLE &&                           \
-      lp == log2_radix(R) * (SP) && tw == 1)                                            \
+      lp == log2_radix(R) * (SP))                                                       \
     return prec == 5 ? launch_pass_t<R, 5, S, log2_radix(R) * (SO), ROLE,               \
                                      log2_radix(R) * (SP)>(a, num_sms, st)              \
                      : launch_pass_t<R, 4, S, log2_radix(R) * (SO), ROLE,               \
                                      log2_radix(R) * (SP)>(a, num_sms, st);
 #define TCU_BF16_TEAM_CASE(S, SO, ROLE, SP, TW)                                         \
   if (s == S && lo == log2_radix(R) * (SO) && role == ROLE &&                           \
-      lp == log2_radix(R) * (SP) && tw == TW)                                           \
+      lp == log2_radix(R) * (SP))                                                       \
     return prec == 5 ? launch_team_t<R, 5, S, log2_radix(R) * (SO), ROLE,               \
                                      log2_radix(R) * (SP), TW>(a, num_sms, st)          \
                      : launch_team_t<R, 4, S, log2_radix(R) * (SO), ROLE,               \

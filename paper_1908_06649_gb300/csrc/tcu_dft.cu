@@ -130,8 +130,8 @@ int plan_mixed_q(int r, long long n, long long batch, PassPlan pass[kMaxPasses])
   pp.modes[0] = kQF;
   pp.modes[1] = kUF;
   pp.modes[2] = kUF;
-  pp.tw = 1;
-  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, 1);
+  pp.tw = team_size(r, pp);
+  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   return 2;
 }
 
@@ -178,18 +178,23 @@ int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]) {
     pp.modes[0] = pp.role == kFirst ? kUF : kQF;
     pp.modes[1] = kUF;
     pp.modes[2] = kUF;
-    pp.tw = 1;
-    pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, 1);
+    pp.tw = team_size(r, pp);
+    pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   }
   return 1 + tc;
 }
 
-// Warpgroups per item of pass pp: 4 for the 3-stage radix-8 passes of
-// two-pass transforms (an item of 512 rows holds 8 sub-transforms of 512
-// points, so the strided side moves 64-byte runs), else 1.
-int team_size(int r, int npasses, const PassPlan &pp) {
-  if (r == 16 && npasses == 1 && pp.s == 3) return 2;
-  return (r == 8 && npasses == 2 && pp.s == 3 && pp.role != kCols) ? 4 : 1;
+// Warpgroups per item of pass pp: 4 for the 3-stage radix-8 passes with a
+// strided side (an item of 512 rows holds 8 sub-transforms of 512 points, so
+// that side moves 64-byte runs; items of one warpgroup move 16-byte runs, half
+// a sector: 8^7 x 32 last pass 567 -> 229 us, 8^8 x 4 passes 2 and 3
+// 562 + 629 -> 271 + 225 us, 512^2 x 200 463 -> 378 us).  After a prefix of
+// two a run is 16 bytes either way: one warpgroup (2 8^3 x 65536: 274 us
+// against 322).  2 for 16^3 in one pass, else 1.
+int team_size(int r, const PassPlan &pp) {
+  if (r == 16 && pp.role == kSingle && pp.s == 3) return 2;
+  if (r != 8 || pp.s != 3 || pp.role == kSingle) return 1;
+  return pp.role == kSecond && pp.lo == 1 ? 1 : 4;
 }
 
 // Role, neighbouring stage counts, size and row maps of pass `pi`.
@@ -218,7 +223,7 @@ void pass_geometry(PassPlan &pp, int pi, int P, const int st[kMaxPasses], int k,
   pp.modes[0] = pp.role == kFirst ? kUF : kQF;
   pp.modes[1] = kUF;
   pp.modes[2] = pp.role == kSingle ? kRQF : kUF;
-  pp.tw = team_size(r, P, pp);
+  pp.tw = team_size(r, pp);
   pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
 }
 
@@ -251,22 +256,18 @@ void free_plan(tcu_dft_plan_s *p) {
 
 // ---------------------------------------------------------------- launches
 cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, int num_sms,
-                          cudaStream_t st, bool team_plan) {
+                          cudaStream_t st) {
   if (pp.mixed) {
     if (r == 8) return launch_pass_mixed_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
     if (r == 16) return launch_pass_mixed_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
     return launch_pass_mixed_r32(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   }
   if (prec_bf16(prec)) {
-    if (r == 8) return launch_pass_bf16_r8(prec, pp.s, pp.lo, pp.role, pp.lp, pp.tw, a, num_sms, st);
+    if (r == 8) return launch_pass_bf16_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
     if (r == 16)
-      return launch_pass_bf16_r16(prec, pp.s, pp.lo, pp.role, pp.lp, pp.tw, a, num_sms, st);
-    return launch_pass_bf16_r32(prec, pp.s, pp.lo, pp.role, pp.lp, pp.tw, a, num_sms, st);
+      return launch_pass_bf16_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
+    return launch_pass_bf16_r32(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   }
-  if (r == 8 && team_plan)
-    return launch_team_r8(prec, pp.s, pp.lo, pp.role, pp.lp, pp.tw, a, num_sms, st);
-  if (r == 16 && pp.tw > 1)
-    return launch_team_r16(prec, pp.s, pp.lo, pp.role, pp.lp, pp.tw, a, num_sms, st);
   if (r == 8) return launch_pass_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   if (r == 16) return launch_pass_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   return launch_pass_r32(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
@@ -421,9 +422,7 @@ int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
     }
     g.bimg = p->bimg[di];
     g.err = p->err;
-    bool team_plan = false;
-    for (int i = 0; i < p->npasses; ++i) team_plan |= p->pass[i].tw > 1;
-    if (pass_dispatch(p->r, p->precision, pp, g, p->num_sms, st, team_plan) != cudaSuccess)
+    if (pass_dispatch(p->r, p->precision, pp, g, p->num_sms, st) != cudaSuccess)
       return TCU_DFT_ERR_CUDA;
   }
   if (events && cudaEventRecord((cudaEvent_t)events[p->npasses], st) != cudaSuccess)

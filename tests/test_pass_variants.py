@@ -1,0 +1,62 @@
+"""GPU parity of the pass variants at the edges of their items: short last
+items, one transform, a batch that no item size divides, the shortest other
+side.  Bar: per-transform relative L2 <= 1e-5 (3xTF32) / 3e-3 (TF32) against
+the fp64 oracle, the bars of the other parity tests."""
+import numpy as np
+import pytest
+
+import inputs
+import oracle
+from oracle import grid
+
+pytestmark = pytest.mark.gpu
+
+TOL = {3: 1e-5, 1: 3e-3, 4: 2e-2, 5: 1e-4}
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    from paper_1908_06649_gb300 import _build
+    _build.build()
+    import paper_1908_06649_gb300 as p
+    p.lib()
+    return p
+
+
+def _check_1d(pkg, n, batch, r, prec, inverse, seed):
+    import torch
+    x = inputs.make("normal", n, batch, seed=seed)
+    plan = pkg.Plan(n, batch, r, prec)
+    xd = torch.from_numpy(x).cuda()
+    y = plan.inverse(xd) if inverse else plan.forward(xd)
+    plan.check()
+    plan.exec(xd, xd, pkg.INVERSE if inverse else pkg.FORWARD)  # in place
+    plan.check()
+    assert torch.equal(xd, y)
+    err = oracle.rel_l2(y.cpu().numpy(), oracle.dft(x, inverse=inverse, threads=8))
+    assert np.all(err <= TOL[prec]), "max rel L2 %.3e" % err.max()
+    plan.destroy()
+
+
+# radix 8, three stages on a strided side: items of four warpgroups hold 8
+# sub-transforms, so 1, 3, 7 and 9 of them leave a short last item
+@pytest.mark.parametrize("n,batch", [(3 * 512, 1), (5 * 512, 2), (7 * 512, 1), (9 * 512, 3),
+                                     (15 * 512, 7), (4 * 512, 1), (4 * 512, 5), (2 * 512, 3),
+                                     (8 ** 5, 1), (8 ** 6, 1), (8 ** 7, 1)])
+@pytest.mark.parametrize("inverse", [False, True])
+def test_radix8_team_items(pkg, n, batch, inverse):
+    _check_1d(pkg, n, batch, 8, 3, inverse, seed=n % 97)
+
+
+@pytest.mark.parametrize("n1,n2,batch", [(512, 8, 1), (512, 64, 3), (512, 512, 1)])
+def test_radix8_team_columns(pkg, n1, n2, batch):
+    import torch
+    x = inputs.make("normal", n1 * n2, batch, seed=5).reshape(batch, n1, n2)
+    plan = pkg.Plan2(n1, n2, batch, 8, 3)
+    y = plan.forward(torch.from_numpy(x).cuda().reshape(-1))
+    plan.check()
+    yh = y.cpu().numpy().reshape(batch, -1)
+    ref = grid.dft2(x, threads=8).reshape(batch, -1)
+    err = np.linalg.norm(yh - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.max() <= TOL[3]
+    plan.destroy()
