@@ -20,31 +20,37 @@ using namespace tcu::host;
 // =========================================================== 2-D transforms
 // A 2-D DFT of batch row-major n1 x n2 arrays (Sec. 4.6: the 1-D DFT of
 // every column, then of every row) is two warpgroup passes: the column pass
-// (kCols: kFirst's strided geometry without a twiddle, T[b][k1][v]) and the
+// (kCols: the strided geometry without a twiddle, T[b][k1][v]) and the
 // row pass (kSingle over batch * n1 rows, natural order).  A circular
 // convolution with a fixed array whose spectrum S is given is three:
 // columns, rows (forward, times S, inverse -- on chip, one item at a time),
 // inverse columns (1/(n1 n2) folded into the last stage's F images).
 
 
-// Axes beyond one warpgroup pass (or the BF16 modes): the general path.
-// The rows of every array are one batched 1-D plan of length n2 (several
-// passes where needed); the arrays are transposed so that the columns are
-// contiguous, transformed by a 1-D plan of length n1 and transposed back.
-// A convolution multiplies by the spectrum on the transposed layout (the
-// spectrum transposed once per call into a plan buffer) between the forward
-// and the inverse column plans.
+// Axes beyond one warpgroup pass, and the BF16 modes (the general path): the
+// columns in up to three strided passes of role kCols (the four-step split of
+// the column length; the digit reversal is in their output rows, so nothing is
+// transposed), then the rows by a 1-D plan of length n2.  HBM-bound: one round
+// trip per pass, two fewer than with a transpose each way (4096 x 4096 x 4
+// 929 -> 568 us, 256 x 256 x 1000 in BF16 788 -> 345, 65536 x 16 x 64
+// 1519 -> 777).  A convolution
+// multiplies by the spectrum as the forward rows are stored (in a pass of its
+// own when the rows need several), then runs the inverse rows and columns.
+// Arrays smaller than one column item (n1 n2 < 128 r) transpose instead:
+// rows, transpose, the columns as rows, transpose back.
 struct tcu_dft2_plan_s {
   long long n1, n2, batch;
   int r, precision, num_sms;
-  PassPlan cols, rows;
-  float *bimg[2];     // [dir index]; scaled copies by 2^-log2(n1 n2)
+  PassPlan rows;
+  float *bimg[2];     // [dir index]; scaled copies by 2^-log2(n1 n2), by 1/n1 (general path)
   float *cimg;        // convolution rows: forward hi, lo | inverse hi, lo
   float2 *scratch;    // batch * n1 * n2
   int *err;
+  int ncol;  // column passes (0: transpose instead)
+  PassPlan colp[kMaxPasses];
   bool general;
-  tcu_dft_plan_t rows1d, cols1d;  // general path: length n2 / n1 plans
-  float2 *spec_t;                 // general path: the spectrum transposed
+  tcu_dft_plan_t rows1d, cols1d;  // length n2 / n1 plans (cols1d: ncol = 0)
+  float2 *spec_t;                 // ncol = 0: the spectrum transposed
 };
 
 struct tcu_stencil_plan_s {
@@ -81,21 +87,18 @@ void free_dft2(tcu_dft2_plan_s *p) {
   tcu_dft_destroy(p->cols1d);
   cudaFree(p->spec_t);
   for (int d = 0; d < 2; ++d) {
+    for (int i = 0; i < p->ncol; ++i) {
+      cudaFree(p->colp[i].tw_stage[d]);
+      cudaFree(p->colp[i].tw_a[d]);
+      cudaFree(p->colp[i].tw_b[d]);
+    }
     cudaFree(p->bimg[d]);
-    cudaFree(p->cols.tw_stage[d]);
     cudaFree(p->rows.tw_stage[d]);
   }
   cudaFree(p->cimg);
   cudaFree(p->scratch);
   cudaFree(p->err);
   delete p;
-}
-
-// Column-pass TMA map: [array][row a][column v], GG columns x n1 rows.
-bool cols_map(CUtensorMap *m, const void *in, const tcu_dft2_plan_s *p) {
-  const long long gg = (128ll * p->cols.tw * p->r) / p->n1;
-  return encode_map(m, in, p->n2, p->n1, p->batch, p->n1 * p->n2, (int)gg,
-                    p->n1 < 256 ? (int)p->n1 : 256);
 }
 
 PRun dft2_pass(const tcu_dft2_plan_s *p, const PassPlan &pp, int di, const float2 *in,
@@ -108,23 +111,48 @@ PRun dft2_pass(const tcu_dft2_plan_s *p, const PassPlan &pp, int di, const float
   g.U = pp.U;
   g.tw_stage = pp.tw_stage[di];
   g.swz_tab = pp.swz_tab;
-  g.last_img = scaled ? 2 * 16 * p->r * p->r : 0;
+  g.last_img = scaled ? 2 * (prec_bf16(p->precision) ? 8 : 16) * p->r * p->r : 0;
   g.spec = spec;
   g.spec_mask = p->n1 - 1;
   g.reverse = reverse;
   return g;
 }
 
-int run_dft2_pass(const tcu_dft2_plan_s *p, const PassPlan &pp, int di, const float2 *in,
-                  float2 *out, bool scaled, const float2 *spec, cudaStream_t st) {
+// The row pass of the two-pass path; it follows the column pass: items last to
+// first (L2 reuse).
+int run_rows(const tcu_dft2_plan_s *p, int di, const float2 *in, float2 *out, bool scaled,
+             cudaStream_t st) {
   GArgs g;
   memset(&g, 0, sizeof(g));
-  // the row pass follows the column pass: items last to first (L2 reuse)
-  g.p[0] = dft2_pass(p, pp, di, in, out, scaled, spec, pp.role == kCols ? 0 : 1);
-  if (pp.role == kCols && !cols_map(&g.tm_in, in, p)) return TCU_DFT_ERR_CUDA;
+  g.p[0] = dft2_pass(p, p->rows, di, in, out, scaled, nullptr, 1);
   g.bimg = p->bimg[di];
   g.err = p->err;
-  return pass_dispatch(p->r, p->precision, pp, g, p->num_sms, st) == cudaSuccess
+  return pass_dispatch(p->r, p->precision, p->rows, g, p->num_sms, st) == cudaSuccess
+             ? TCU_DFT_OK
+             : TCU_DFT_ERR_CUDA;
+}
+
+// Column pass i; scaled: with the scaled F images.
+int run_col_pass(const tcu_dft2_plan_s *p, int i, int di, const float2 *in, float2 *out,
+                 bool scaled, cudaStream_t st) {
+  const PassPlan &c = p->colp[i];
+  GArgs g;
+  memset(&g, 0, sizeof(g));
+  // every second pass last to first (L2 reuse), as in the 1-D plans
+  g.p[0] = dft2_pass(p, c, di, in, out, scaled, nullptr, (i & 1) && c.tw == 1);
+  g.p[0].lo = c.lo;
+  g.p[0].lp = c.lp;
+  g.p[0].lc = ilog2(p->n2);
+  g.p[0].tw_out = c.tw_a[di];
+  g.p[0].tw_b = c.tw_b[di];
+  const long long L = 1ll << c.log2L;
+  const int gg = (int)((128ll * c.tw * p->r) >> c.log2L);
+  if (!encode_map(&g.tm_in, in, 1ll << c.lo, L, p->batch << c.lp, L << c.lo, gg,
+                  L < 256 ? (int)L : 256))
+    return TCU_DFT_ERR_CUDA;
+  g.bimg = p->bimg[di];
+  g.err = p->err;
+  return pass_dispatch(p->r, p->precision, c, g, p->num_sms, st) == cudaSuccess
              ? TCU_DFT_OK
              : TCU_DFT_ERR_CUDA;
 }
@@ -135,10 +163,85 @@ int check_buffers(const void *in, const void *out, size_t bytes) {
   return TCU_DFT_OK;
 }
 
-// The general path: 1-D plans for the rows (n2, batch n1 of them) and the
-// columns (n1, batch n2 of them), a scratch array and the transposed
-// spectrum of a convolution.  UNSUPPORTED if either length has no 1-D plan.
-tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_t r,
+// Stages of the strided passes of columns of length r^k beside n2 columns, as
+// plan_stages but with at most two radix-16 stages each.  Every item's columns
+// must exist: GG <= rest n2.  0: no such split (transpose instead).
+int col_stages(int r, int k, long long n2, int st[kMaxPasses]) {
+  int P;
+  if (k <= single_pass_stages(r)) {
+    st[0] = k;
+    P = 1;
+  } else if (r == 16 && k == 3) {
+    st[0] = 1;
+    st[1] = 2;
+    P = 2;
+  } else if (r == 8 && k == 4 && n2 < 16) {
+    st[0] = 1;  // a 2-stage item spans 16 columns, a 3-stage team item 8
+    st[1] = 3;
+    P = 2;
+  } else {
+    P = plan_stages(r, k, st);
+  }
+  long long rest = n2;
+  for (int i = P - 1; i >= 0; --i) {
+    const long long L = 1ll << (ilog2(r) * st[i]);
+    const int tw = r == 8 && st[i] == 3 ? 4 : 1;
+    if (rest * L < 128ll * tw * r) return 0;
+    rest *= L;
+  }
+  return P;
+}
+
+// The columns' tables: the F images scaled by 1/n, and per column pass
+// its geometry, stage twiddles and inter-pass twiddles [row of rest][k].
+int make_cols(tcu_dft2_plan_s *p, const int *st, long long n) {
+  const int log2r = ilog2(p->r);
+  int rc = TCU_DFT_OK;
+  long long pre = 1;
+  for (int i = 0; i < p->ncol; ++i) {
+    PassPlan &c = p->colp[i];
+    const long long L = 1ll << (log2r * st[i]), rest = p->n1 / (pre * L);
+    c.s = st[i];
+    c.role = kCols;
+    c.log2L = log2r * c.s;
+    c.lo = ilog2(rest * p->n2);
+    c.lp = ilog2(pre);
+    c.last = i == p->ncol - 1;
+    c.U = p->batch * pre * rest * p->n2;
+    c.modes[0] = c.modes[1] = c.modes[2] = kUF;
+    c.tw = team_size(p->r, c);
+    c.swz_tab = choose_swizzle(p->r, c.s, c.modes, c.tw);
+    for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
+      const int sign = d == 0 ? -1 : 1;
+      rc = upload(&c.tw_stage[d], stage_twiddles(p->r, c.s, sign));
+      if (c.last || rc != TCU_DFT_OK) continue;
+      // [row of rest][k], in two levels beyond kColRows rows
+      const long long low = rest >> kLog2ColRows ? 1ll << kLog2ColRows : rest;
+      std::vector<float2> t((size_t)(low * L));
+      for (long long a = 0; a < low; ++a)
+        for (long long k = 0; k < L; ++k) t[(size_t)(a * L + k)] = root(a * k, L * rest, sign);
+      rc = upload(&c.tw_a[d], t);
+      if (low == rest || rc != TCU_DFT_OK) continue;
+      t.resize((size_t)(rest / low * L));
+      for (long long a = 0; a < rest / low; ++a)
+        for (long long k = 0; k < L; ++k)
+          t[(size_t)(a * L + k)] = root(a * low * k, L * rest, sign);
+      rc = upload(&c.tw_b[d], t);
+    }
+    pre *= L;
+  }
+  for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
+    std::vector<float> img;
+    build_images(p->r, d == 0 ? -1 : 1, n, p->precision, img);
+    rc = upload(&p->bimg[d], img);
+  }
+  return rc;
+}
+
+// The general path: the rows by a 1-D plan (n2, batch n1 of them), the columns
+// by strided passes, or (small arrays) by a 1-D plan between transposes.
+// UNSUPPORTED if either length has no 1-D plan.
+tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_t r, int k1,
                                    int32_t precision, int &rc) {
   // both lengths must have a 1-D plan (a host-side question: no CUDA call)
   int32_t st[kMaxPasses];
@@ -154,9 +257,12 @@ tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_
   p->r = r;
   p->precision = precision;
   p->general = true;
+  int cst[kMaxPasses];
+  p->ncol = col_stages(r, k1, n2, cst);
   p->rows1d = tcu_dft_plan(n2, batch * n1, r, precision);
   rc = p->rows1d ? TCU_DFT_OK : tcu_dft_last_error();
-  if (rc == TCU_DFT_OK) {
+  if (rc == TCU_DFT_OK && p->ncol) rc = make_cols(p, cst, n1);
+  if (rc == TCU_DFT_OK && !p->ncol) {
     p->cols1d = tcu_dft_plan(n1, batch * n2, r, precision);
     rc = p->cols1d ? TCU_DFT_OK : tcu_dft_last_error();
   }
@@ -164,7 +270,8 @@ tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_
     p->num_sms = p->rows1d->num_sms;
     if (dev_malloc((void **)&p->scratch, (size_t)(batch * n1 * n2) * sizeof(float2)) !=
             cudaSuccess ||
-        dev_malloc((void **)&p->spec_t, (size_t)(n1 * n2) * sizeof(float2)) != cudaSuccess ||
+        (!p->ncol &&
+         dev_malloc((void **)&p->spec_t, (size_t)(n1 * n2) * sizeof(float2)) != cudaSuccess) ||
         dev_malloc((void **)&p->err, sizeof(int)) != cudaSuccess ||
         cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
@@ -178,22 +285,80 @@ tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_
   return p;
 }
 
-// General path: the 2-D transform of `in` into `out` (rows, transpose,
-// columns, transpose back), or -- with keep_t -- left transposed in the
-// plan's scratch after the columns (the convolution continues there).
-int general_dft2(const tcu_dft2_plan_s *p, const void *in, void *out, int dir, bool keep_t,
+// The column passes from `in` (the plan's scratch, out or the caller's input),
+// alternating between `out` and the scratch, never in place; `src` is left at
+// the result.
+int run_cols(const tcu_dft2_plan_s *p, int di, const float2 *&src, float2 *out,
+             cudaStream_t st) {
+  for (int i = 0; i < p->ncol; ++i) {
+    float2 *dst = src == p->scratch ? out : p->scratch;
+    const int rc = run_col_pass(p, i, di, src, dst, di == 1 && p->colp[i].last, st);
+    if (rc != TCU_DFT_OK) return rc;
+    src = dst;
+  }
+  return TCU_DFT_OK;
+}
+
+// General path: the 2-D transform of `in` into `out`.
+int general_dft2(const tcu_dft2_plan_s *p, const void *in, void *out, int dir,
                  cudaStream_t st) {
+  const int di = dir_index(dir);
+  if (p->ncol) {
+    const float2 *src = (const float2 *)in;
+    const int rc = run_cols(p, di, src, (float2 *)out, st);
+    return rc != TCU_DFT_OK ? rc : tcu_dft_exec_dir(p->rows1d, src, out, dir, st);
+  }
   int rc = tcu_dft_exec_dir(p->rows1d, in, out, dir, st);
   if (rc != TCU_DFT_OK) return rc;
   if (launch_transpose(p->scratch, (const float2 *)out, p->batch, p->n1, p->n2, p->num_sms,
                        st) != cudaSuccess)
     return TCU_DFT_ERR_CUDA;
   rc = tcu_dft_exec_dir(p->cols1d, p->scratch, p->scratch, dir, st);
-  if (rc != TCU_DFT_OK || keep_t) return rc;
+  if (rc != TCU_DFT_OK) return rc;
   return launch_transpose((float2 *)out, p->scratch, p->batch, p->n2, p->n1, p->num_sms, st) ==
                  cudaSuccess
              ? TCU_DFT_OK
              : TCU_DFT_ERR_CUDA;
+}
+
+// General path: the convolution of `in` with the array of the given spectrum.
+int general_conv2(const tcu_dft2_plan_s *p, const void *in, const float2 *spectrum, void *out,
+                  cudaStream_t st) {
+  if (p->ncol) {
+    // columns; rows forward, times the spectrum; rows and columns back
+    const float2 *src = (const float2 *)in;
+    int rc = run_cols(p, 0, src, (float2 *)out, st);
+    if (rc != TCU_DFT_OK) return rc;
+    float2 *at = const_cast<float2 *>(src);  // the scratch or out
+    const bool fused = p->rows1d->npasses == 1;
+    rc = exec_impl(p->rows1d, at, at, TCU_DFT_FORWARD, st, nullptr, 0, 0, -1,
+                   fused ? spectrum : nullptr, p->n1 - 1);
+    if (rc != TCU_DFT_OK) return rc;
+    if (!fused && launch_spectrum_product(at, spectrum, p->batch, p->n1 * p->n2, p->num_sms,
+                                          st) != cudaSuccess)
+      return TCU_DFT_ERR_CUDA;
+    rc = exec_impl(p->rows1d, at, at, TCU_DFT_INVERSE, st, nullptr);
+    return rc != TCU_DFT_OK ? rc : run_cols(p, 1, src, (float2 *)out, st);
+  }
+  // rows and columns forward (left transposed in the scratch), times the
+  // spectrum transposed, columns back, transpose back, rows back
+  int rc = tcu_dft_exec_dir(p->rows1d, in, out, TCU_DFT_FORWARD, st);
+  if (rc != TCU_DFT_OK) return rc;
+  if (launch_transpose(p->scratch, (const float2 *)out, p->batch, p->n1, p->n2, p->num_sms,
+                       st) != cudaSuccess)
+    return TCU_DFT_ERR_CUDA;
+  rc = tcu_dft_exec_dir(p->cols1d, p->scratch, p->scratch, TCU_DFT_FORWARD, st);
+  if (rc != TCU_DFT_OK) return rc;
+  if (launch_transpose(p->spec_t, spectrum, 1, p->n1, p->n2, p->num_sms, st) != cudaSuccess ||
+      launch_spectrum_product(p->scratch, p->spec_t, p->batch, p->n1 * p->n2, p->num_sms, st) !=
+          cudaSuccess)
+    return TCU_DFT_ERR_CUDA;
+  rc = tcu_dft_exec_dir(p->cols1d, p->scratch, p->scratch, TCU_DFT_INVERSE, st);
+  if (rc != TCU_DFT_OK) return rc;
+  if (launch_transpose((float2 *)out, p->scratch, p->batch, p->n2, p->n1, p->num_sms, st) !=
+      cudaSuccess)
+    return TCU_DFT_ERR_CUDA;
+  return tcu_dft_exec_dir(p->rows1d, out, out, TCU_DFT_INVERSE, st);
 }
 
 tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
@@ -214,7 +379,7 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   // TF32 modes: the two-pass path; otherwise the general path
   if (prec_bf16(precision) || k1 > single_pass_stages(r) || k2 > single_pass_stages(r) ||
       n1 * n2 < 128ll * r)
-    return make_dft2_general(n1, n2, batch, r, precision, rc);
+    return make_dft2_general(n1, n2, batch, r, k1, precision, rc);
   int dev = 0;
   cudaDeviceProp prop;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess ||
@@ -232,18 +397,7 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   p->precision = precision;
   p->num_sms = prop.multiProcessorCount;
   const int log2r = ilog2(r);
-  PassPlan &c = p->cols, &w = p->rows;
-  c.s = k1;
-  c.role = kCols;
-  c.so = k2;
-  c.sp = 0;
-  c.lo = log2r * k2;
-  c.lp = 0;
-  c.log2L = log2r * k1;
-  c.U = batch * n2;
-  c.modes[0] = c.modes[1] = c.modes[2] = kUF;
-  c.tw = team_size(r, c);
-  c.swz_tab = choose_swizzle(r, c.s, c.modes, c.tw);
+  PassPlan &w = p->rows;
   w.s = k2;
   w.role = kSingle;
   w.so = w.sp = w.lo = w.lp = 0;
@@ -255,15 +409,15 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   w.tw = team_size(r, w);
   w.swz_tab = choose_swizzle(r, w.s, w.modes, w.tw);
   std::vector<float> conv_img;
+  p->ncol = 1;
+  rc = make_cols(p, &k1, n1 * n2);
   for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
     const int sign = d == 0 ? -1 : 1;
     std::vector<float> img;
     build_images(r, sign, n1 * n2, precision, img);
-    rc = upload(&p->bimg[d], img);
     // hi and lo of this direction (the first two images)
     conv_img.insert(conv_img.end(), img.begin(), img.begin() + img.size() / 2);
-    if (rc == TCU_DFT_OK) rc = upload(&c.tw_stage[d], stage_twiddles(r, c.s, sign));
-    if (rc == TCU_DFT_OK) rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, sign));
+    rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, sign));
   }
   if (rc == TCU_DFT_OK) rc = upload(&p->cimg, conv_img);
   if (rc == TCU_DFT_OK &&
@@ -344,15 +498,14 @@ int tcu_dft2_exec(tcu_dft2_plan_t p, const void *in, void *out, int dir, void *s
   const int di = dir_index(dir);
   if (p->general) {
     const NvtxRange range("tcu_dft2 (general)");
-    rc = general_dft2(p, in, out, dir, false, st);
+    rc = general_dft2(p, in, out, dir, st);
     return rc == TCU_DFT_OK && debug_exec() ? tcu_dft2_check(p, stream) : rc;
   }
   {
     const NvtxRange range("tcu_dft2");
-    rc = run_dft2_pass(p, p->cols, di, (const float2 *)in, p->scratch, false, nullptr, st);
+    rc = run_col_pass(p, 0, di, (const float2 *)in, p->scratch, false, st);
     if (rc == TCU_DFT_OK)
-      rc = run_dft2_pass(p, p->rows, di, p->scratch, (float2 *)out, dir == TCU_DFT_INVERSE,
-                         nullptr, st);
+      rc = run_rows(p, di, p->scratch, (float2 *)out, dir == TCU_DFT_INVERSE, st);
   }
   return rc == TCU_DFT_OK && debug_exec() ? tcu_dft2_check(p, stream) : rc;
 }
@@ -366,27 +519,13 @@ int tcu_conv2_exec(tcu_dft2_plan_t p, const void *in, const void *spectrum, void
   cudaStream_t st = (cudaStream_t)stream;
   const NvtxRange range("tcu_conv2");
   if (p->general) {
-    // forward rows and columns (left transposed in the scratch), times the
-    // spectrum transposed, inverse columns, transpose back, inverse rows
-    rc = general_dft2(p, in, out, TCU_DFT_FORWARD, true, st);
-    if (rc != TCU_DFT_OK) return rc;
-    if (launch_transpose(p->spec_t, (const float2 *)spectrum, 1, p->n1, p->n2, p->num_sms,
-                         st) != cudaSuccess ||
-        launch_spectrum_product(p->scratch, p->spec_t, p->batch, p->n1 * p->n2, p->num_sms,
-                                st) != cudaSuccess)
-      return TCU_DFT_ERR_CUDA;
-    rc = tcu_dft_exec_dir(p->cols1d, p->scratch, p->scratch, TCU_DFT_INVERSE, st);
-    if (rc != TCU_DFT_OK) return rc;
-    if (launch_transpose((float2 *)out, p->scratch, p->batch, p->n2, p->n1, p->num_sms, st) !=
-        cudaSuccess)
-      return TCU_DFT_ERR_CUDA;
-    rc = tcu_dft_exec_dir(p->rows1d, out, out, TCU_DFT_INVERSE, st);
+    rc = general_conv2(p, in, (const float2 *)spectrum, out, st);
     return rc == TCU_DFT_OK && debug_exec() ? tcu_dft2_check(p, stream) : rc;
   }
   // columns: in -> scratch; rows forward, times the spectrum and inverse on
   // chip: scratch -> scratch (an item reads its rows before writing them);
   // inverse columns with 1/(n1 n2): scratch -> out
-  rc = run_dft2_pass(p, p->cols, 0, (const float2 *)in, p->scratch, false, nullptr, st);
+  rc = run_col_pass(p, 0, 0, (const float2 *)in, p->scratch, false, st);
   if (rc != TCU_DFT_OK) return rc;
   GArgs g;
   memset(&g, 0, sizeof(g));
@@ -399,7 +538,7 @@ int tcu_conv2_exec(tcu_dft2_plan_t p, const void *in, const void *spectrum, void
   else if (p->r == 16) e = launch_rowconv_r16(p->precision, p->rows.s, g, p->num_sms, st);
   else e = launch_rowconv_r32(p->precision, p->rows.s, g, p->num_sms, st);
   if (e != cudaSuccess) return TCU_DFT_ERR_CUDA;
-  rc = run_dft2_pass(p, p->cols, 1, p->scratch, (float2 *)out, true, nullptr, st);
+  rc = run_col_pass(p, 0, 1, p->scratch, (float2 *)out, true, st);
   return rc == TCU_DFT_OK && debug_exec() ? tcu_dft2_check(p, stream) : rc;
 }
 
@@ -407,7 +546,7 @@ int tcu_dft2_check(tcu_dft2_plan_t p, void *stream) {
   if (!p) return TCU_DFT_ERR_INVALID;
   if (p->general) {
     int rc = tcu_dft_check(p->rows1d, stream);
-    if (rc == TCU_DFT_OK) rc = tcu_dft_check(p->cols1d, stream);
+    if (rc == TCU_DFT_OK && p->cols1d) rc = tcu_dft_check(p->cols1d, stream);
     if (rc != TCU_DFT_OK) return rc;
   }
   if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return TCU_DFT_ERR_CUDA;

@@ -59,7 +59,9 @@ enum RowMode { kQF = 0, kUF = 1, kRQF = 2 };
 // kSecondQ: the last pass of a mixed-radix transform n = q R^S whose factor
 // q (2 .. 16, any integer) is a runtime value: the q-point first pass's
 // output T[b n + v L + a], v < q, -> y[b n + v + k q]
-enum Role { kSingle = 0, kFirst = 1, kSecond = 2, kCols = 3, kSecondQ = 4 };
+// kCols: one of several column passes of a 2-D transform, whose column
+// count, prefix and remaining rows are runtime values
+enum Role { kSingle = 0, kFirst = 1, kSecond = 2, kSecondQ = 4, kCols = 5 };
 
 __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 16 ? 4 : 5); }
 // Warpgroups per CTA: TMEM holds 512 columns, a warpgroup's slot 3 Q of
@@ -73,7 +75,8 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // radix-16 first (strided) pass also stages its inter-pass twiddles
 // in SMEM, which leaves room for four; a radix-16 last pass of several runs
 // four too (measured faster than five: 0.165 instead of 0.181 ms for the
-// second pass of n = 16^4 x 1024).  A radix-32 pass of two stages runs
+// second pass of n = 16^4 x 1024), and so does a column pass (256 x 256 x
+// 1000 339 us against 363).  A radix-32 pass of two stages runs
 // four warpgroups whose slots hold A for half of K (the products of a stage
 // in two K halves); one-stage radix-32 passes (already near the copy rate),
 // the convolution row pass and the fused schedule keep whole-K slots, two
@@ -81,7 +84,7 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 __host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
   return R == 8    ? (S == 3 ? 5 : 8)
          : R == 32 ? (S >= 2 ? 4 : 2)
-                   : ((ROLE == 1 || ROLE == 2) && R == 16 ? 4 : 5);
+                   : (ROLE != 0 && ROLE != 4 ? 4 : 5);
 }
 __host__ __device__ constexpr int whole_k_nwg(int R, int ROLE, int S = 2) {
   return R == 32 ? 2 : pass_nwg(R, ROLE, S);
@@ -100,9 +103,14 @@ __host__ __device__ constexpr int team_nwg(int R) { return R == 8 ? 8 : 4; }
 //            transform.  Sequence b' = (b, p), p < P, holds z[b' M + a n2 + v];
 //            the DFT over a, times w_M^{v k}, goes to T[b n + (k P + p) n2 + v]
 //            (for LP = 0: T[b n + k n2 + v])
-//   kCols  : the column pass of a 2-D DFT of n1 x n2 arrays (n1 = R^S,
-//            n2 = 2^LO): kFirst's geometry with LP = 0 and no twiddle,
-//            x[b n + a n2 + v] -> X[b n + k n2 + v]
+//   kCols : pass of the columns of n1 x n2 arrays with n1 = P L rest (P
+//            rows' digits transformed before, rest after): sequence (b, p)
+//            holds z[(p L rest) n2 + a rest n2 + v], v = (row of rest,
+//            column) < rest n2 = 2^lo; the DFT over a goes to row (k P + p) of
+//            rest n2 values, times w_{L rest}^{k (v / n2)} unless it is the
+//            last (LP = 1: with the twiddle, 0: without).  lo, log2 P and
+//            log2 n2 are PRun::lo, lp, lc: the strides are shifts, and an
+//            array of any shape needs one kernel per radix and stage count
 //   kSecond: last of several passes, n1 = 2^LO points before it per row:
 //            T[b n + v L + a] -> y[b n + v + k n1]
 //
@@ -127,6 +135,8 @@ struct Geo {
   static constexpr int L = 1 << LOG2L;
   static constexpr int LOG2N = LOG2R * S + LO;          // sequence length M
   static constexpr int LOG2PRE = ROLE == kFirst ? LP : 0;
+  // runtime column geometry (PRun::lo, lp, lc), with twiddle
+  static constexpr bool RTC = ROLE == kCols, RTC_TW = RTC && LP == 1;
   static constexpr int LOG2NT = LOG2N + LOG2PRE;        // transform length n
   static constexpr int LOG2RPS = LOG2L - LOG2R;   // rows per sub-transform
   static constexpr int LOG2GG = LOG2GPTS - LOG2L; // sub-transforms per item
@@ -136,7 +146,7 @@ struct Geo {
   static constexpr long long OUT_STRIDE =
       ROLE == kSingle ? 1 : (1ll << (LOG2O + LOG2PRE));
   static constexpr long long OUT_VSTRIDE = ROLE == kSingle ? 0 : 1;
-  static constexpr bool STRIDED = ROLE == kFirst || ROLE == kCols;
+  static constexpr bool STRIDED = ROLE == kFirst || RTC;
   // the sub-transforms' prefix count q is a runtime value (PRun::q)
   static constexpr bool RTQ = ROLE == kSecondQ;
   static constexpr int MODE_FIRST = STRIDED ? kUF : kQF;
@@ -165,10 +175,13 @@ struct Geo {
   static constexpr int TW_ENTRIES = S == 1 ? 0 : (S == 2 ? R * R : R * R * R + R * R);
   static_assert(LOG2GG >= 0, "sub-transform longer than one item");
   static_assert(LOG2GG <= LOG2VL || !TW_OUT, "an item spans one twiddle column block");
-  static_assert(LOG2GG <= LOG2UPER || !STRIDED, "an item spans columns of one sequence");
+  static_assert(LOG2GG <= LOG2UPER || !STRIDED || RTC, "an item spans columns of one sequence");
   static_assert(NWG * GCOLS <= 512, "TMEM budget");
   static_assert(NTEAM * TW == NWG && (TW == 1 || TW == 2 || TW == 4), "team size");
 };
+
+// Rows of a column pass's one-level twiddle table.
+constexpr int kLog2ColRows = 10;
 
 // Runtime part of a pass.
 struct PRun {
@@ -191,6 +204,10 @@ struct PRun {
   int reverse;
   // kSecondQ: the factor q of n = q R^S (sub-transforms per transform)
   int q;
+  // kCols: log2 of the values after a row (rest n2), of the prefix P and of
+  // the columns n2; its twiddles are tw_out[row of rest][k] (rows beyond
+  // kColRows: tw_out[row mod kColRows][k] times tw_b[row / kColRows][k])
+  int lo, lp, lc;
 };
 
 struct GArgs {
@@ -246,6 +263,12 @@ struct SmemLayout {
   static constexpr size_t BYTES = OFF_SCHED + 32 * NWG;
   static_assert(BYTES <= 227 * 1024, "shared memory budget");
 };
+
+// log2 of the sub-transforms per sequence.
+template <class G>
+__device__ __forceinline__ int log2_uper(const PRun &P) {
+  return G::RTC ? P.lo : G::LOG2UPER;
+}
 
 // Per-warpgroup state.
 struct WG {
@@ -471,8 +494,8 @@ __device__ __forceinline__ void issue_input(const PRun &P, const CUtensorMap *tm
   const uint32_t dst = smem_u32(w.stg);
   if (G::MODE_FIRST == kUF) {
     // strided first pass: box of GG sub-transforms x L points
-    const long long b = u0 >> G::LOG2UPER;
-    const int v0 = (int)(u0 & ((1ll << G::LOG2UPER) - 1));
+    const long long b = u0 >> log2_uper<G>(P);
+    const int v0 = (int)(u0 & ((1ll << log2_uper<G>(P)) - 1));
     if (elect_one()) {
       mbar_expect_tx(w.bar_stg, G::GPTS * 8);
 #pragma unroll
@@ -682,8 +705,8 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
     klow = (klow << G::LOG2R) | (vq & (R - 1));
     vq >>= G::LOG2R;
   }
-  long long b = u >> G::LOG2UPER;
-  long long v = u & ((1ll << G::LOG2UPER) - 1);
+  long long b = u >> log2_uper<G>(P);
+  long long v = u & ((1ll << log2_uper<G>(P)) - 1);
   // kFirst after a prefix: sequence b = (transform, p) -> transform-major,
   // k above p
   const long long bt = b >> G::LOG2PRE, bp = b & ((1ll << G::LOG2PRE) - 1);
@@ -698,6 +721,22 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
     dst = P.out + b * (q << G::LOG2L) + v + klow * q;
     JS = q << (G::LOG2L - G::LOG2R);
   }
+  if constexpr (G::RTC) {
+    // sequence b = (array, p): row (k P + p) of the array
+    const int ls = P.lo + P.lp;
+    dst = P.out + ((b >> P.lp) << (ls + G::LOG2L)) + ((b & ((1ll << P.lp) - 1)) << P.lo) + v +
+          ((long long)klow << ls);
+    JS = 1ll << (ls + G::LOG2L - G::LOG2R);
+  }
+  // kCols twiddles [row of rest][k]: k runs across lanes, so a warp reads a
+  // few sectors, mostly the same ones as its SM's other warpgroups
+  const long long crow = v >> P.lc;
+  const long long coff = ((crow & ((1 << kLog2ColRows) - 1)) << G::LOG2L) + klow;
+  const long long cboff = ((crow >> kLog2ColRows) << G::LOG2L) + klow;
+  const int lrest = P.lo - P.lc;
+  const long long c_elems = (long long)G::L << min(lrest, kLog2ColRows);
+  const long long cb_elems = (long long)G::L << max(lrest - kLog2ColRows, 0);
+  const bool ctwo = G::RTC_TW && P.tw_b != nullptr;
   // twiddle of output k = klow + j r^(S-1): table A staged as [k][ul] in SMEM,
   // or read from global [k][vl]; two-level: times B[vh][k]
   const float2 *tws = w.tws + klow * G::GG + ul;
@@ -731,6 +770,11 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
       if (G::MODE_LAST == kRQF && mul)
         fs[jj] = in_range(w, soff + j * JS, (P.spec_mask + 1) << G::LOG2L) ? __ldg(sp + j * JS)
                                                                           : one;
+      if (G::RTC_TW) {
+        fa[jj] = in_range(w, coff + j * TBJ, c_elems) ? __ldg(P.tw_out + coff + j * TBJ) : one;
+        if (ctwo && in_range(w, cboff + j * TBJ, cb_elems))
+          fa[jj] = cmul(fa[jj], __ldg(P.tw_b + cboff + j * TBJ));
+      }
       if (G::TW_SMEM) {
         fa[jj] = in_range(w, toff + j * TJS, G::GPTS) ? tws[j * TJS] : one;
         if (G::TW2L) fb[jj] = in_range(w, klow + j * TBJ, G::L) ? twbs[j * TBJ] : one;
@@ -748,6 +792,7 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
       const int j = c + jj;
       float2 y = make_float2(d[2 * j], d[2 * j + 1]);
       if (G::MODE_LAST == kRQF && mul) y = cmul(y, fs[jj]);
+      if (G::RTC_TW) y = cmul(y, fa[jj]);
       if (G::TW_SMEM || G::TW_OUT) y = G::TW2L ? cmul(y, cmul(fa[jj], fb[jj])) : cmul(y, fa[jj]);
       if (in_range(w, doff + j * JS, out_elems)) {
         if (OUT_L2)
@@ -1277,7 +1322,7 @@ __global__ void __launch_bounds__(
       // a strided pass writes the next pass's input: L2-cached stores keep
       // its latest part for the next pass (which starts there), streaming
       // stores otherwise
-      process_item<G, PREC, ROLE == kFirst>(P, &a.tm_tw, tw, phys(item), w, nx);
+      process_item<G, PREC, ROLE == kFirst || ROLE == kCols>(P, &a.tm_tw, tw, phys(item), w, nx);
     item += istride;
   }
   if (w.fail && w.rho == 0) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);

@@ -210,10 +210,13 @@ void dir_tables(const tcu_dft_plan_s *p, int d, DirTables &t);
 // The transform of transforms [b0, b0 + count) of the plan's batch (in and
 // out point at transform b0; count < 0: the whole batch).  The intermediates
 // of that range sit at the same offset in the plan's scratch, so disjoint
-// ranges may run concurrently on different streams (not fused plans).
+// ranges may run concurrently on different streams (not fused plans).  spec:
+// for a plan of one pass, transform b is multiplied by the spectrum row
+// spec[(b & spec_mask) n ...] as it is stored (the rows of a 2-D convolution).
 int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
                      void *stream, void *const *events, long long queue_start = 0,
-                     long long b0 = 0, long long count = -1);
+                     long long b0 = 0, long long count = -1, const float2 *spec = nullptr,
+                     long long spec_mask = 0);
 
 }  // namespace host
 }  // namespace tcu

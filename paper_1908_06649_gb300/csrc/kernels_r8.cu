@@ -27,12 +27,6 @@ cudaError_t launch_pass_r8(int prec, int s, int lo, int role, int lp, const GArg
   TCU_TEAM_CASE(3, 6, kFirst, 0, 4)   // n = 8^9: 3 + 3 + 3
   TCU_TEAM_CASE(3, 3, kFirst, 3, 4)
   TCU_TEAM_CASE(3, 6, kSecond, 0, 4)
-  TCU_PASS_CASE(1, 3, kCols, 0)   // 2-D DFT column passes: n1 = R^s, n2 = R^so
-  TCU_PASS_CASE(2, 2, kCols, 0)
-  TCU_PASS_CASE(2, 3, kCols, 0)
-  TCU_TEAM_CASE(3, 1, kCols, 0, 4)
-  TCU_TEAM_CASE(3, 2, kCols, 0, 4)
-  TCU_TEAM_CASE(3, 3, kCols, 0, 4)
   return cudaErrorInvalidValue;
 }
 

@@ -8,7 +8,7 @@
 namespace tcu {
 
 // One warpgroup pass of radix 8, 16 or 32: s stages, role kSingle / kFirst /
-// kSecond / kCols; lo = log2 of the columns of a strided pass or of the
+// kSecond; lo = log2 of the columns of a strided pass or of the
 // points before a last pass; lp = log2 of the prefix count of a strided pass.
 // cudaErrorInvalidValue for a combination that is not instantiated.
 cudaError_t launch_pass_r8(int prec, int s, int lo, int role, int lp, const GArgs &a,
@@ -17,6 +17,15 @@ cudaError_t launch_pass_r16(int prec, int s, int lo, int role, int lp, const GAr
                             int num_sms, cudaStream_t st);
 cudaError_t launch_pass_r32(int prec, int s, int lo, int role, int lp, const GArgs &a,
                             int num_sms, cudaStream_t st);
+// A column pass of a 2-D transform whose columns need several passes, or of a
+// BF16 mode (kernels_cols_r*.cu): s stages, twid: with the inter-pass twiddle;
+// the shape is in a.p[0].lo, lp, lc.
+cudaError_t launch_cols_r8(int prec, int s, int twid, const GArgs &a, int num_sms,
+                           cudaStream_t st);
+cudaError_t launch_cols_r16(int prec, int s, int twid, const GArgs &a, int num_sms,
+                            cudaStream_t st);
+cudaError_t launch_cols_r32(int prec, int s, int twid, const GArgs &a, int num_sms,
+                            cudaStream_t st);
 // The row pass of a circular 2-D convolution: each row transformed,
 // multiplied by the spectrum and transformed back on chip (s stages).
 cudaError_t launch_rowconv_r8(int prec, int s, const GArgs &a, int num_sms, cudaStream_t st);

@@ -140,6 +140,16 @@ cudaError_t launch_pair_t(const GArgs &a, int clusters, cudaStream_t st) {
                                      log2_radix(R) * (SP), TW>(a, num_sms, st)          \
                      : launch_team_t<R, 4, S, log2_radix(R) * (SO), ROLE,               \
                                      log2_radix(R) * (SP), TW>(a, num_sms, st);
+// A column pass of a 2-D transform (kCols) of S stages, with (TWID = 1) or
+// without its inter-pass twiddle, items of TW warpgroups; every precision.
+#define TCU_COLS_CASE(S, TWID, LAUNCH, ...)                                              \
+  if (s == S && twid == TWID) {                                                          \
+    if (prec == 3) return LAUNCH<R, 3, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
+    if (prec == 1) return LAUNCH<R, 1, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
+    if (prec == 5) return LAUNCH<R, 5, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
+    return LAUNCH<R, 4, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);                 \
+  }
+#define TCU_COMMA ,
 #define TCU_FUSED_CASE(S1, S2)                                                      \
   if (s1 == S1 && s2 == S2)                                                         \
     return prec == 3 ? launch_fused_t<R, 3, S1, S2>(a, num_sms, st)                 \

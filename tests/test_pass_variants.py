@@ -48,15 +48,49 @@ def test_radix8_team_items(pkg, n, batch, inverse):
     _check_1d(pkg, n, batch, 8, 3, inverse, seed=n % 97)
 
 
-@pytest.mark.parametrize("n1,n2,batch", [(512, 8, 1), (512, 64, 3), (512, 512, 1)])
-def test_radix8_team_columns(pkg, n1, n2, batch):
+# column passes of a runtime shape: one, two and three of them, the fewest
+# columns an item spans, a two-level twiddle table (2^20 rows), a batch that
+# leaves the last items to few warpgroups, every precision
+@pytest.mark.parametrize("r,n1,n2,batch,prec", [
+    (8, 512, 8, 1, 3), (8, 512, 64, 3, 3), (8, 512, 512, 1, 5), (8, 4096, 8, 2, 3),
+    (8, 4096, 64, 1, 4), (8, 8, 512, 3, 5), (16, 16, 256, 7, 5), (16, 256, 16, 3, 4),
+    (16, 4096, 16, 2, 3), (16, 4096, 16, 1, 1), (16, 1 << 20, 16, 1, 3), (32, 1024, 32, 1, 5),
+    (32, 32768, 32, 1, 4), (32, 32, 1024, 3, 1)])
+@pytest.mark.parametrize("inverse", [False, True])
+def test_column_passes(pkg, r, n1, n2, batch, prec, inverse):
     import torch
     x = inputs.make("normal", n1 * n2, batch, seed=5).reshape(batch, n1, n2)
-    plan = pkg.Plan2(n1, n2, batch, 8, 3)
-    y = plan.forward(torch.from_numpy(x).cuda().reshape(-1))
+    plan = pkg.Plan2(n1, n2, batch, r, prec)
+    d = pkg.INVERSE if inverse else pkg.FORWARD
+    xd = torch.from_numpy(x).cuda()
+    y = plan.exec(xd, None, d)
+    plan.check()
+    assert torch.equal(plan.exec(xd, xd, d), y)  # in place
     plan.check()
     yh = y.cpu().numpy().reshape(batch, -1)
-    ref = grid.dft2(x, threads=8).reshape(batch, -1)
+    ref = grid.dft2(x, inverse=inverse, threads=8).reshape(batch, -1)
     err = np.linalg.norm(yh - ref, axis=1) / np.linalg.norm(ref, axis=1)
-    assert err.max() <= TOL[3]
+    assert err.max() <= TOL[prec]
+    plan.destroy()
+
+
+# a convolution is two transforms and a product: twice the bar of one (the
+# spectrum is given in fp32; the product's rounding is far below)
+@pytest.mark.parametrize("r,n1,n2,batch,prec", [
+    (16, 256, 4096, 2, 5), (16, 256, 256, 3, 4), (8, 4096, 8, 3, 3), (8, 64, 4096, 1, 3),
+    (32, 1024, 1024, 1, 5), (16, 16, 65536, 2, 3)])
+def test_column_passes_conv(pkg, r, n1, n2, batch, prec):
+    import torch
+    x = inputs.make("uniform", n1 * n2, batch, seed=6).reshape(batch, n1, n2)
+    w = inputs.make("normal", n1 * n2, 1, seed=7).reshape(n1, n2)
+    plan = pkg.Plan2(n1, n2, batch, r, prec)
+    xd, wd = torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda()
+    y = plan.conv(xd, wd)
+    plan.check()
+    assert torch.equal(plan.conv(xd, wd, xd), y)
+    plan.check()
+    ref = torch.fft.ifft2(torch.fft.fft2(torch.from_numpy(x).cdouble())
+                          * torch.from_numpy(w).cdouble()).numpy().reshape(batch, -1)
+    err = np.linalg.norm(y.cpu().numpy().reshape(batch, -1) - ref, axis=1)
+    assert (err / np.linalg.norm(ref, axis=1)).max() <= 2 * TOL[prec]
     plan.destroy()
