@@ -47,6 +47,40 @@ __global__ void cpow_kernel(float2 *g, long long count, int k) {
   }
 }
 
+// Rows f1 = 0 .. N / 2 of the spectrum of Lemma 1's kernel W' on an N x N
+// periodic grid, directly: w[-a mod N][-b mod N] = W[k + a][k + b] are the
+// coefficients of P^k (Lemma 2), so its DFT at (f1, f2) is P(x, y)^k with
+// x = w_N^{-f1}, y = w_N^{-f2} (N >= 2 k + 1: nothing wraps).  In fp64, rounded
+// once: the k-th power multiplies a relative error of P by k.  A few dozen
+// fp64 operations a point and one launch, where placing P, its transform, the
+// power, the inverse, placing W' and its transform were nine (40 us).
+__global__ void stencil_spectrum_kernel(float2 *S, const double2 *roots, int N, Stencil3 w,
+                                        int k) {
+  const int count = (N / 2 + 1) * N;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
+    const double2 x = roots[e / N], y = roots[e % N];  // w_N^{-f}
+    double2 r[3];  // sum over b of w[a][b] y^b
+    for (int a = 0; a < 3; ++a) {
+      const double lo = w.w[3 * a], hi = w.w[3 * a + 2];
+      r[a] = make_double2(fma(lo + hi, y.x, (double)w.w[3 * a + 1]), (hi - lo) * y.y);
+    }
+    // x^-1 r[0] + r[1] + x r[2]
+    double2 base;
+    base.x = fma(x.x, r[0].x + r[2].x, fma(x.y, r[0].y - r[2].y, r[1].x));
+    base.y = fma(x.x, r[0].y + r[2].y, fma(x.y, r[2].x - r[0].x, r[1].y));
+    double2 acc = make_double2(1.0, 0.0);
+    for (int m = k;;) {
+      if (m & 1)
+        acc = make_double2(fma(acc.x, base.x, -acc.y * base.y),
+                           fma(acc.x, base.y, acc.y * base.x));
+      m >>= 1;
+      if (!m) break;
+      base = make_double2(fma(base.x, base.x, -base.y * base.y), 2.0 * base.x * base.y);
+    }
+    S[e] = make_float2((float)acc.x, (float)acc.y);
+  }
+}
+
 // W[(k + a)(2k + 1) + (k + b)] = Re g[a mod Nw][b mod Nw], |a|, |b| <= k.
 __global__ void extract_weights_kernel(float *W, const float2 *g, long long Nw, int k) {
   const long long side = 2 * k + 1, count = side * side;
@@ -177,6 +211,17 @@ cudaError_t launch_place_poly(float2 *g, long long Nw, const Stencil3 &w, int nu
 
 cudaError_t launch_cpow(float2 *g, long long count, int k, int num_sms, cudaStream_t st) {
   cpow_kernel<<<grid_for(count, num_sms), kBlock, 0, st>>>(g, count, k);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_stencil_spectrum(float2 *S, const double2 *roots, long long N,
+                                    const Stencil3 &w, int k, int num_sms, cudaStream_t st) {
+  // one point per thread in small blocks, over all SMs (their few fp64 units
+  // bound it)
+  const long long blocks = ((N / 2 + 1) * N + 63) / 64;
+  const long long cap = 16ll * num_sms;
+  stencil_spectrum_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 64, 0, st>>>(S, roots,
+                                                                                 (int)N, w, k);
   return cudaGetLastError();
 }
 

@@ -28,14 +28,14 @@ using namespace tcu::host;
 
 
 // Axes beyond one warpgroup pass, and the BF16 modes (the general path): the
-// columns in up to three strided passes of role kCols (the four-step split of
-// the column length; the digit reversal is in their output rows, so nothing is
-// transposed), then the rows by a 1-D plan of length n2.  HBM-bound: one round
-// trip per pass, two fewer than with a transpose each way (4096 x 4096 x 4
-// 929 -> 568 us, 256 x 256 x 1000 in BF16 788 -> 345, 65536 x 16 x 64
-// 1519 -> 777).  A convolution
-// multiplies by the spectrum as the forward rows are stored (in a pass of its
-// own when the rows need several), then runs the inverse rows and columns.
+// rows by a 1-D plan of length n2, then the columns in up to three strided
+// passes of role kCols (the four-step split of the column length; the digit
+// reversal is in their output rows, so nothing is transposed).  HBM-bound: one
+// round trip per pass, two fewer than with a transpose each way (4096 x 4096 x 4
+// 929 -> 562 us, 256 x 256 x 1000 in BF16 788 -> 335, 65536 x 16 x 64
+// 1519 -> 766).  A
+// convolution multiplies by the spectrum as the last forward column pass
+// stores, then runs the inverse columns and rows.
 // Arrays smaller than one column item (n1 n2 < 128 r) transpose instead:
 // rows, transpose, the columns as rows, transpose back.
 struct tcu_dft2_plan_s {
@@ -53,17 +53,37 @@ struct tcu_dft2_plan_s {
   float2 *spec_t;                 // ncol = 0: the spectrum transposed
 };
 
+// A stencil plan.  In 3xTF32 with tiles of one warpgroup pass per axis the
+// tiles stay real (`real`): the column pass gathers them from the grid, two
+// real columns as one complex one (N / 2 columns a tile); the row pass
+// untangles the rows 0 .. N / 2 of the column spectra (the others are their
+// conjugates), convolves them and packs them again; the inverse column pass
+// scatters the output blocks to the grid.  Half the transforms and a third of
+// the traffic of complex tiles (4096^2, 16 steps: 378 -> 153 us; 512^2 radix-8
+// tiles, 100 steps: 1053 -> 454).  The other modes keep complex
+// tiles: with single products every rounding of the operands would move.
 struct tcu_stencil_plan_s {
   long long side, N, Nw, tiles;
   int B;  // output block side: N - 2k (Lemma 1's tiles are blocks of k)
   int k, r, precision, num_sms;
-  tcu_dft2_plan_t conv;   // N x N, batch = tiles
-  tcu_dft2_plan_t wconv;  // N x N, batch 1 (spectrum of the kernel)
+  bool real;              // real tiles
+  bool closed;            // the spectrum by stencil_spectrum_kernel
+  tcu_dft2_plan_t conv;   // N x N (real: N x N / 2), batch = tiles
+  tcu_dft2_plan_t wconv;  // N x N, batch 1 (spectrum of the kernel; not closed)
   tcu_dft2_plan_t wpow;   // Nw x Nw, batch 1 (Lemma 2)
-  float2 *tile_buf;       // tiles * N * N
+  float2 *tile_buf;       // tiles * N * N (not real)
   float2 *wgrid;          // Nw * Nw
   float2 *wker;           // N * N: the kernel W', then its spectrum
+  double2 *roots;         // closed: w_N^{-f}, f < N
 };
+
+// Steps up to which a real-tile plan evaluates the kernel's spectrum directly:
+// one launch instead of nine (a grid of 1000^2, 16 steps: 114 -> 45 us), and
+// more exact (error of the output 7.9e-6 -> 1.3e-6).  Beyond, the spectrum
+// comes from the transforms of Lemma 2, as tcu_stencil_weights' weights do:
+// their error grows with k (about 5e-7 k of the output), and results stay
+// within 2e-5 of theirs on either side of the line.
+constexpr int kClosedSteps = 24;
 
 namespace {
 
@@ -132,14 +152,14 @@ int run_rows(const tcu_dft2_plan_s *p, int di, const float2 *in, float2 *out, bo
              : TCU_DFT_ERR_CUDA;
 }
 
-// Column pass i; scaled: with the scaled F images.
+// Column pass i; scaled: with the scaled F images; spec: its output times this
+// spectrum (last pass); reverse: items last to first.
 int run_col_pass(const tcu_dft2_plan_s *p, int i, int di, const float2 *in, float2 *out,
-                 bool scaled, cudaStream_t st) {
+                 bool scaled, const float2 *spec, bool reverse, cudaStream_t st) {
   const PassPlan &c = p->colp[i];
   GArgs g;
   memset(&g, 0, sizeof(g));
-  // every second pass last to first (L2 reuse), as in the 1-D plans
-  g.p[0] = dft2_pass(p, c, di, in, out, scaled, nullptr, (i & 1) && c.tw == 1);
+  g.p[0] = dft2_pass(p, c, di, in, out, scaled, spec, reverse && c.tw == 1);
   g.p[0].lo = c.lo;
   g.p[0].lp = c.lp;
   g.p[0].lc = ilog2(p->n2);
@@ -152,7 +172,8 @@ int run_col_pass(const tcu_dft2_plan_s *p, int i, int di, const float2 *in, floa
     return TCU_DFT_ERR_CUDA;
   g.bimg = p->bimg[di];
   g.err = p->err;
-  return pass_dispatch(p->r, p->precision, c, g, p->num_sms, st) == cudaSuccess
+  const int mode = !c.last ? kColTwiddle : (spec ? kColSpectrum : kColPlain);
+  return launch_cols(p->r, p->precision, c.s, mode, g, p->num_sms, st) == cudaSuccess
              ? TCU_DFT_OK
              : TCU_DFT_ERR_CUDA;
 }
@@ -166,7 +187,7 @@ int check_buffers(const void *in, const void *out, size_t bytes) {
 // Stages of the strided passes of columns of length r^k beside n2 columns, as
 // plan_stages but with at most two radix-16 stages each.  Every item's columns
 // must exist: GG <= rest n2.  0: no such split (transpose instead).
-int col_stages(int r, int k, long long n2, int st[kMaxPasses]) {
+int col_stages(int r, int k, long long n2, int precision, int st[kMaxPasses]) {
   int P;
   if (k <= single_pass_stages(r)) {
     st[0] = k;
@@ -176,7 +197,10 @@ int col_stages(int r, int k, long long n2, int st[kMaxPasses]) {
     st[1] = 2;
     P = 2;
   } else if (r == 8 && k == 4 && n2 < 16) {
-    st[0] = 1;  // a 2-stage item spans 16 columns, a 3-stage team item 8
+    // a 2-stage item spans 16 columns, a 3-stage team item 8; the other split
+    // rounds the operands of the single-product modes elsewhere
+    if (precision != TCU_DFT_3XTF32) return 0;
+    st[0] = 1;
     st[1] = 3;
     P = 2;
   } else {
@@ -258,7 +282,7 @@ tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_
   p->precision = precision;
   p->general = true;
   int cst[kMaxPasses];
-  p->ncol = col_stages(r, k1, n2, cst);
+  p->ncol = col_stages(r, k1, n2, precision, cst);
   p->rows1d = tcu_dft_plan(n2, batch * n1, r, precision);
   rc = p->rows1d ? TCU_DFT_OK : tcu_dft_last_error();
   if (rc == TCU_DFT_OK && p->ncol) rc = make_cols(p, cst, n1);
@@ -285,16 +309,18 @@ tcu_dft2_plan_s *make_dft2_general(int64_t n1, int64_t n2, int64_t batch, int32_
   return p;
 }
 
-// The column passes from `in` (the plan's scratch, out or the caller's input),
-// alternating between `out` and the scratch, never in place; `src` is left at
-// the result.
-int run_cols(const tcu_dft2_plan_s *p, int di, const float2 *&src, float2 *out,
+// The column passes of one direction on `at`, one of the scratch and `out`,
+// alternating between the two; returns a status and leaves `at` at the result.
+int run_cols(const tcu_dft2_plan_s *p, int di, float2 *&at, float2 *out, const float2 *spec,
              cudaStream_t st) {
   for (int i = 0; i < p->ncol; ++i) {
-    float2 *dst = src == p->scratch ? out : p->scratch;
-    const int rc = run_col_pass(p, i, di, src, dst, di == 1 && p->colp[i].last, st);
+    float2 *dst = at == p->scratch ? out : p->scratch;
+    const bool last = p->colp[i].last;
+    // every second pass last to first, from the rows' pass on (L2 reuse)
+    const int rc = run_col_pass(p, i, di, at, dst, di == 1 && last, last ? spec : nullptr,
+                                !(i & 1), st);
     if (rc != TCU_DFT_OK) return rc;
-    src = dst;
+    at = dst;
   }
   return TCU_DFT_OK;
 }
@@ -302,11 +328,12 @@ int run_cols(const tcu_dft2_plan_s *p, int di, const float2 *&src, float2 *out,
 // General path: the 2-D transform of `in` into `out`.
 int general_dft2(const tcu_dft2_plan_s *p, const void *in, void *out, int dir,
                  cudaStream_t st) {
-  const int di = dir_index(dir);
   if (p->ncol) {
-    const float2 *src = (const float2 *)in;
-    const int rc = run_cols(p, di, src, (float2 *)out, st);
-    return rc != TCU_DFT_OK ? rc : tcu_dft_exec_dir(p->rows1d, src, out, dir, st);
+    // the column passes alternate and end in out
+    float2 *at = p->ncol & 1 ? p->scratch : (float2 *)out;
+    const int rc = tcu_dft_exec_dir(p->rows1d, in, at, dir, st);
+    return rc != TCU_DFT_OK ? rc
+                            : run_cols(p, dir_index(dir), at, (float2 *)out, nullptr, st);
   }
   int rc = tcu_dft_exec_dir(p->rows1d, in, out, dir, st);
   if (rc != TCU_DFT_OK) return rc;
@@ -325,20 +352,12 @@ int general_dft2(const tcu_dft2_plan_s *p, const void *in, void *out, int dir,
 int general_conv2(const tcu_dft2_plan_s *p, const void *in, const float2 *spectrum, void *out,
                   cudaStream_t st) {
   if (p->ncol) {
-    // columns; rows forward, times the spectrum; rows and columns back
-    const float2 *src = (const float2 *)in;
-    int rc = run_cols(p, 0, src, (float2 *)out, st);
-    if (rc != TCU_DFT_OK) return rc;
-    float2 *at = const_cast<float2 *>(src);  // the scratch or out
-    const bool fused = p->rows1d->npasses == 1;
-    rc = exec_impl(p->rows1d, at, at, TCU_DFT_FORWARD, st, nullptr, 0, 0, -1,
-                   fused ? spectrum : nullptr, p->n1 - 1);
-    if (rc != TCU_DFT_OK) return rc;
-    if (!fused && launch_spectrum_product(at, spectrum, p->batch, p->n1 * p->n2, p->num_sms,
-                                          st) != cudaSuccess)
-      return TCU_DFT_ERR_CUDA;
-    rc = exec_impl(p->rows1d, at, at, TCU_DFT_INVERSE, st, nullptr);
-    return rc != TCU_DFT_OK ? rc : run_cols(p, 1, src, (float2 *)out, st);
+    // rows and columns forward, times the spectrum, columns and rows back
+    float2 *at = (float2 *)out;
+    int rc = tcu_dft_exec_dir(p->rows1d, in, out, TCU_DFT_FORWARD, st);
+    if (rc == TCU_DFT_OK) rc = run_cols(p, 0, at, (float2 *)out, spectrum, st);
+    if (rc == TCU_DFT_OK) rc = run_cols(p, 1, at, (float2 *)out, nullptr, st);
+    return rc != TCU_DFT_OK ? rc : tcu_dft_exec_dir(p->rows1d, out, out, TCU_DFT_INVERSE, st);
   }
   // rows and columns forward (left transposed in the scratch), times the
   // spectrum transposed, columns back, transpose back, rows back
@@ -361,6 +380,129 @@ int general_conv2(const tcu_dft2_plan_s *p, const void *in, const float2 *spectr
   return tcu_dft_exec_dir(p->rows1d, out, out, TCU_DFT_INVERSE, st);
 }
 
+// Plans run on sm_103 only; the number of its SMs.
+int device_sms(int &rc) {
+  int dev = 0;
+  cudaDeviceProp prop;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess ||
+      prop.major != 10 || prop.minor != 3) {
+    cudaGetLastError();
+    rc = TCU_DFT_ERR_CUDA;
+    return 0;
+  }
+  rc = TCU_DFT_OK;
+  return prop.multiProcessorCount;
+}
+
+// Tables and buffers of the two-pass path: rows of row_len points (U of them) in
+// one pass, the columns of n1 x n2 arrays in another; images scaled by
+// 1 / (n1 row_len).
+int make_two_pass(tcu_dft2_plan_s *p, int k1, int k2, long long row_len, long long U) {
+  const int r = p->r;
+  PassPlan &w = p->rows;
+  w.s = k2;
+  w.role = kSingle;
+  w.so = w.sp = w.lo = w.lp = 0;
+  w.log2L = ilog2(r) * k2;
+  w.U = U;
+  w.modes[0] = kQF;
+  w.modes[1] = kUF;
+  w.modes[2] = kRQF;
+  w.tw = team_size(r, w);
+  w.swz_tab = choose_swizzle(r, w.s, w.modes, w.tw);
+  std::vector<float> conv_img;
+  p->ncol = 1;
+  int rc = make_cols(p, &k1, p->n1 * row_len);
+  for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
+    const int sign = d == 0 ? -1 : 1;
+    std::vector<float> img;
+    build_images(r, sign, p->n1 * row_len, p->precision, img);
+    // hi and lo of this direction (the first two images)
+    conv_img.insert(conv_img.end(), img.begin(), img.begin() + img.size() / 2);
+    rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, sign));
+  }
+  if (rc == TCU_DFT_OK) rc = upload(&p->cimg, conv_img);
+  if (rc == TCU_DFT_OK &&
+      (dev_malloc((void **)&p->scratch, (size_t)(p->batch * p->n1 * p->n2) * sizeof(float2)) !=
+           cudaSuccess ||
+       dev_malloc((void **)&p->err, sizeof(int)) != cudaSuccess ||
+       cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess)) {
+    cudaGetLastError();
+    rc = TCU_DFT_ERR_OOM;
+  }
+  return rc;
+}
+
+// The passes of `tiles` real N x N tiles (N = r^k, 3xTF32): packed arrays of
+// N x N / 2.
+tcu_dft2_plan_s *make_real_tiles(int64_t N, int k, int64_t tiles, int32_t r, int &rc) {
+  const int sms = device_sms(rc);
+  if (rc != TCU_DFT_OK) return nullptr;
+  tcu_dft2_plan_s *p = new tcu_dft2_plan_s();
+  memset(p, 0, sizeof(*p));
+  p->n1 = N;
+  p->n2 = N / 2;
+  p->batch = tiles;
+  p->r = r;
+  p->precision = TCU_DFT_3XTF32;
+  p->num_sms = sms;
+  rc = make_two_pass(p, k, k, N, tiles * (N / 2 + 1));
+  if (rc != TCU_DFT_OK) {
+    free_dft2(p);
+    return nullptr;
+  }
+  return p;
+}
+
+cudaError_t launch_rowconv(const tcu_dft2_plan_s *p, bool real, const GArgs &g,
+                           cudaStream_t st) {
+  if (p->r == 8) return launch_rowconv_r8(p->precision, p->rows.s, real, g, p->num_sms, st);
+  if (p->r == 16) return launch_rowconv_r16(p->precision, p->rows.s, real, g, p->num_sms, st);
+  return launch_rowconv_r32(p->precision, p->rows.s, real, g, p->num_sms, st);
+}
+
+// Convolve every tile of the grid A with the kernel of the given spectrum (rows
+// 0 .. N / 2 of it) into the output blocks of Ak: three launches.
+int run_real_tiles(const tcu_stencil_plan_s *sp, const float *A, float *Ak,
+                   const float2 *spectrum, cudaStream_t st) {
+  const tcu_dft2_plan_s *p = sp->conv;
+  const PassPlan &c = p->colp[0];
+  GArgs g;
+  memset(&g, 0, sizeof(g));
+  g.err = p->err;
+  for (int pass = 0; pass < 3; ++pass) {
+    const int di = pass == 2 ? 1 : 0;
+    // the row pass runs last to first, so each pass starts on what the one
+    // before wrote last
+    g.p[0] = pass == 1 ? dft2_pass(p, p->rows, 0, p->scratch, p->scratch, false, spectrum, 1)
+                       : dft2_pass(p, c, di, p->scratch, p->scratch, pass == 2, nullptr);
+    PRun &q = g.p[0];
+    q.lo = q.lc = c.lo;
+    q.grid_in = A;
+    q.grid_out = Ak;
+    q.side = sp->side;
+    q.tpr = (int)((sp->side + sp->B - 1) / sp->B);
+    q.block = sp->B;
+    q.halo = sp->k;
+    q.half = (int)(sp->N / 2 + 1);
+    g.bimg = pass == 1 ? p->cimg : p->bimg[di];
+    g.p[1].tw_stage = p->rows.tw_stage[1];
+    cudaError_t e;
+    if (pass == 1) {
+      e = launch_rowconv(p, true, g, st);
+    } else {
+      const int gg = (int)((128ll * c.tw * p->r) >> c.log2L);
+      if (pass == 2 && !encode_map(&g.tm_in, p->scratch, p->n2, p->n1, p->batch, p->n1 * p->n2,
+                                   gg, p->n1 < 256 ? (int)p->n1 : 256))
+        return TCU_DFT_ERR_CUDA;
+      e = launch_cols(p->r, p->precision, c.s, pass == 0 ? kColGather : kColScatter, g,
+                      p->num_sms, st);
+    }
+    if (e != cudaSuccess) return TCU_DFT_ERR_CUDA;
+  }
+  return TCU_DFT_OK;
+}
+
 tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
                            int32_t precision, int &rc) {
   rc = TCU_DFT_OK;
@@ -380,14 +522,8 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   if (prec_bf16(precision) || k1 > single_pass_stages(r) || k2 > single_pass_stages(r) ||
       n1 * n2 < 128ll * r)
     return make_dft2_general(n1, n2, batch, r, k1, precision, rc);
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess ||
-      prop.major != 10 || prop.minor != 3) {
-    cudaGetLastError();
-    rc = TCU_DFT_ERR_CUDA;
-    return nullptr;
-  }
+  const int sms = device_sms(rc);
+  if (rc != TCU_DFT_OK) return nullptr;
   tcu_dft2_plan_s *p = new tcu_dft2_plan_s();
   memset(p, 0, sizeof(*p));
   p->n1 = n1;
@@ -395,39 +531,8 @@ tcu_dft2_plan_s *make_dft2(int64_t n1, int64_t n2, int64_t batch, int32_t r,
   p->batch = batch;
   p->r = r;
   p->precision = precision;
-  p->num_sms = prop.multiProcessorCount;
-  const int log2r = ilog2(r);
-  PassPlan &w = p->rows;
-  w.s = k2;
-  w.role = kSingle;
-  w.so = w.sp = w.lo = w.lp = 0;
-  w.log2L = log2r * k2;
-  w.U = batch * n1;
-  w.modes[0] = kQF;
-  w.modes[1] = kUF;
-  w.modes[2] = kRQF;
-  w.tw = team_size(r, w);
-  w.swz_tab = choose_swizzle(r, w.s, w.modes, w.tw);
-  std::vector<float> conv_img;
-  p->ncol = 1;
-  rc = make_cols(p, &k1, n1 * n2);
-  for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
-    const int sign = d == 0 ? -1 : 1;
-    std::vector<float> img;
-    build_images(r, sign, n1 * n2, precision, img);
-    // hi and lo of this direction (the first two images)
-    conv_img.insert(conv_img.end(), img.begin(), img.begin() + img.size() / 2);
-    rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, sign));
-  }
-  if (rc == TCU_DFT_OK) rc = upload(&p->cimg, conv_img);
-  if (rc == TCU_DFT_OK &&
-      (dev_malloc((void **)&p->scratch, (size_t)(batch * n1 * n2) * sizeof(float2)) !=
-           cudaSuccess ||
-       dev_malloc((void **)&p->err, sizeof(int)) != cudaSuccess ||
-       cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess)) {
-    cudaGetLastError();
-    rc = TCU_DFT_ERR_OOM;
-  }
+  p->num_sms = sms;
+  rc = make_two_pass(p, k1, k2, n2, batch * n1);
   if (rc != TCU_DFT_OK) {
     free_dft2(p);
     return nullptr;
@@ -443,6 +548,7 @@ void free_stencil(tcu_stencil_plan_s *p) {
   cudaFree(p->tile_buf);
   cudaFree(p->wgrid);
   cudaFree(p->wker);
+  cudaFree(p->roots);
   delete p;
 }
 
@@ -503,7 +609,7 @@ int tcu_dft2_exec(tcu_dft2_plan_t p, const void *in, void *out, int dir, void *s
   }
   {
     const NvtxRange range("tcu_dft2");
-    rc = run_col_pass(p, 0, di, (const float2 *)in, p->scratch, false, st);
+    rc = run_col_pass(p, 0, di, (const float2 *)in, p->scratch, false, nullptr, false, st);
     if (rc == TCU_DFT_OK)
       rc = run_rows(p, di, p->scratch, (float2 *)out, dir == TCU_DFT_INVERSE, st);
   }
@@ -525,7 +631,7 @@ int tcu_conv2_exec(tcu_dft2_plan_t p, const void *in, const void *spectrum, void
   // columns: in -> scratch; rows forward, times the spectrum and inverse on
   // chip: scratch -> scratch (an item reads its rows before writing them);
   // inverse columns with 1/(n1 n2): scratch -> out
-  rc = run_col_pass(p, 0, 0, (const float2 *)in, p->scratch, false, st);
+  rc = run_col_pass(p, 0, 0, (const float2 *)in, p->scratch, false, nullptr, false, st);
   if (rc != TCU_DFT_OK) return rc;
   GArgs g;
   memset(&g, 0, sizeof(g));
@@ -533,12 +639,9 @@ int tcu_conv2_exec(tcu_dft2_plan_t p, const void *in, const void *spectrum, void
   g.p[1].tw_stage = p->rows.tw_stage[1];
   g.bimg = p->cimg;
   g.err = p->err;
-  cudaError_t e;
-  if (p->r == 8) e = launch_rowconv_r8(p->precision, p->rows.s, g, p->num_sms, st);
-  else if (p->r == 16) e = launch_rowconv_r16(p->precision, p->rows.s, g, p->num_sms, st);
-  else e = launch_rowconv_r32(p->precision, p->rows.s, g, p->num_sms, st);
+  const cudaError_t e = launch_rowconv(p, false, g, st);
   if (e != cudaSuccess) return TCU_DFT_ERR_CUDA;
-  rc = run_col_pass(p, 0, 1, p->scratch, (float2 *)out, true, st);
+  rc = run_col_pass(p, 0, 1, p->scratch, (float2 *)out, true, nullptr, false, st);
   return rc == TCU_DFT_OK && debug_exec() ? tcu_dft2_check(p, stream) : rc;
 }
 
@@ -594,13 +697,25 @@ tcu_stencil_plan_t tcu_stencil_plan(int64_t side, int32_t steps, int32_t sqrt_m,
   p->B = B;
   p->tiles = tpr * tpr;
   int rc = TCU_DFT_OK;
-  p->conv = make_dft2(N, N, p->tiles, sqrt_m, precision, rc);
-  if (rc == TCU_DFT_OK) p->wconv = make_dft2(N, N, 1, sqrt_m, precision, rc);
+  int kt = 0;
+  is_power_of(N, sqrt_m, kt);
+  p->real = precision == TCU_DFT_3XTF32 && kt <= single_pass_stages(sqrt_m);
+  p->closed = p->real && steps <= kClosedSteps;
+  p->conv = p->real ? make_real_tiles(N, kt, p->tiles, sqrt_m, rc)
+                    : make_dft2(N, N, p->tiles, sqrt_m, precision, rc);
+  if (rc == TCU_DFT_OK && p->closed) {
+    std::vector<double2> roots((size_t)N);
+    for (long long f = 0; f < N; ++f)
+      roots[f] = make_double2(cos(2.0 * M_PI * f / N), sin(2.0 * M_PI * f / N));
+    rc = upload(&p->roots, roots);
+  } else if (rc == TCU_DFT_OK) {
+    p->wconv = make_dft2(N, N, 1, sqrt_m, precision, rc);
+  }
   if (rc == TCU_DFT_OK) p->wpow = make_dft2(Nw, Nw, 1, sqrt_m, precision, rc);
   if (rc == TCU_DFT_OK) {
     p->num_sms = p->conv->num_sms;
-    if (dev_malloc((void **)&p->tile_buf, (size_t)(p->tiles * N * N) * sizeof(float2)) !=
-            cudaSuccess ||
+    if ((!p->real && dev_malloc((void **)&p->tile_buf,
+                                (size_t)(p->tiles * N * N) * sizeof(float2)) != cudaSuccess) ||
         dev_malloc((void **)&p->wgrid, (size_t)(Nw * Nw) * sizeof(float2)) != cudaSuccess ||
         dev_malloc((void **)&p->wker, (size_t)(N * N) * sizeof(float2)) != cudaSuccess) {
       cudaGetLastError();
@@ -646,13 +761,26 @@ int tcu_stencil_exec(tcu_stencil_plan_t p, const float *w3x3, const float *A, fl
   if (A != Ak && overlaps(A, Ak, bytes)) return TCU_DFT_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   const NvtxRange range("tcu_stencil");
-  // W (Lemma 2), the kernel W' and its spectrum
-  int rc = stencil_weight_grid(p, w3x3, st);
-  if (rc != TCU_DFT_OK) return rc;
-  if (launch_place_kernel(p->wker, p->N, p->wgrid, p->Nw, p->k, p->num_sms, st) != cudaSuccess)
-    return TCU_DFT_ERR_CUDA;
-  rc = tcu_dft2_exec(p->wconv, p->wker, p->wker, TCU_DFT_FORWARD, st);
-  if (rc != TCU_DFT_OK) return rc;
+  // the spectrum of W': directly, or W (Lemma 2), the kernel and its transform
+  int rc = TCU_DFT_OK;
+  if (p->closed) {
+    Stencil3 w;
+    for (int i = 0; i < 9; ++i) w.w[i] = w3x3[i];
+    if (launch_stencil_spectrum(p->wker, p->roots, p->N, w, p->k, p->num_sms, st) != cudaSuccess)
+      return TCU_DFT_ERR_CUDA;
+  } else {
+    rc = stencil_weight_grid(p, w3x3, st);
+    if (rc != TCU_DFT_OK) return rc;
+    if (launch_place_kernel(p->wker, p->N, p->wgrid, p->Nw, p->k, p->num_sms, st) !=
+        cudaSuccess)
+      return TCU_DFT_ERR_CUDA;
+    rc = tcu_dft2_exec(p->wconv, p->wker, p->wker, TCU_DFT_FORWARD, st);
+    if (rc != TCU_DFT_OK) return rc;
+  }
+  if (p->real) {
+    rc = run_real_tiles(p, A, Ak, p->wker, st);
+    return rc == TCU_DFT_OK && debug_exec() ? tcu_stencil_check(p, stream) : rc;
+  }
   // Lemma 1: every block's input window as one batch of tiles, circular
   // convolution, the B x B centres
   if (launch_gather_tiles(p->tile_buf, A, p->side, p->k, p->N, p->B, p->num_sms, st) !=
@@ -669,7 +797,7 @@ int tcu_stencil_exec(tcu_stencil_plan_t p, const float *w3x3, const float *A, fl
 int tcu_stencil_check(tcu_stencil_plan_t p, void *stream) {
   if (!p) return TCU_DFT_ERR_INVALID;
   int rc = tcu_dft2_check(p->wpow, stream);
-  if (rc == TCU_DFT_OK) rc = tcu_dft2_check(p->wconv, stream);
+  if (rc == TCU_DFT_OK && p->wconv) rc = tcu_dft2_check(p->wconv, stream);
   if (rc == TCU_DFT_OK) rc = tcu_dft2_check(p->conv, stream);
   return rc;
 }

@@ -62,6 +62,20 @@ enum RowMode { kQF = 0, kUF = 1, kRQF = 2 };
 // kCols: one of several column passes of a 2-D transform, whose column
 // count, prefix and remaining rows are runtime values
 enum Role { kSingle = 0, kFirst = 1, kSecond = 2, kSecondQ = 4, kCols = 5 };
+// What a column pass (the LP argument of a kCols kernel) does besides its
+// transforms: an inter-pass twiddle; a product with a spectrum; input rows
+// gathered as pairs of real columns from the windows of a real grid; output
+// rows scattered back to it.
+enum ColMode {
+  kColPlain = 0,
+  kColTwiddle = 1,
+  kColSpectrum = 2,
+  kColGather = 3,
+  kColScatter = 4
+};
+// Convolution row passes (the CONV argument of a kSingle kernel): of complex
+// arrays, or of real arrays in the packed half-spectrum layout.
+enum ConvMode { kNoConv = 0, kConv = 1, kRealConv = 2 };
 
 __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 16 ? 4 : 5); }
 // Warpgroups per CTA: TMEM holds 512 columns, a warpgroup's slot 3 Q of
@@ -80,14 +94,15 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // four warpgroups whose slots hold A for half of K (the products of a stage
 // in two K halves); one-stage radix-32 passes (already near the copy rate),
 // the convolution row pass and the fused schedule keep whole-K slots, two
-// per CTA at radix 32 (whole_k_nwg).
+// per CTA at radix 32 (whole_k_nwg).  Convolution rows run four at radix 16
+// (registers: 256 x 256 x 500 303 -> 301 us, real tiles 170 -> 167).
 __host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
   return R == 8    ? (S == 3 ? 5 : 8)
          : R == 32 ? (S >= 2 ? 4 : 2)
                    : (ROLE != 0 && ROLE != 4 ? 4 : 5);
 }
 __host__ __device__ constexpr int whole_k_nwg(int R, int ROLE, int S = 2) {
-  return R == 32 ? 2 : pass_nwg(R, ROLE, S);
+  return R == 32 ? 2 : (R == 16 ? 4 : pass_nwg(R, ROLE, S));
 }
 // Warpgroups per CTA of a team pass: two teams of four at radix 8, two teams
 // of two at radix 16 (TMEM: 96 columns a slot; SMEM).
@@ -108,9 +123,9 @@ __host__ __device__ constexpr int team_nwg(int R) { return R == 8 ? 8 : 4; }
 //            holds z[(p L rest) n2 + a rest n2 + v], v = (row of rest,
 //            column) < rest n2 = 2^lo; the DFT over a goes to row (k P + p) of
 //            rest n2 values, times w_{L rest}^{k (v / n2)} unless it is the
-//            last (LP = 1: with the twiddle, 0: without).  lo, log2 P and
-//            log2 n2 are PRun::lo, lp, lc: the strides are shifts, and an
-//            array of any shape needs one kernel per radix and stage count
+//            last.  lo, log2 P and log2 n2 are PRun::lo, lp, lc: the strides
+//            are shifts, and an array of any shape needs one kernel per radix
+//            and stage count.  LP is the pass's ColMode
 //   kSecond: last of several passes, n1 = 2^LO points before it per row:
 //            T[b n + v L + a] -> y[b n + v + k n1]
 //
@@ -136,7 +151,10 @@ struct Geo {
   static constexpr int LOG2N = LOG2R * S + LO;          // sequence length M
   static constexpr int LOG2PRE = ROLE == kFirst ? LP : 0;
   // runtime column geometry (PRun::lo, lp, lc), with twiddle
-  static constexpr bool RTC = ROLE == kCols, RTC_TW = RTC && LP == 1;
+  static constexpr bool RTC = ROLE == kCols, RTC_TW = RTC && LP == kColTwiddle;
+  static constexpr bool RTC_SPEC = RTC && LP == kColSpectrum;
+  static constexpr bool GATHER = RTC && LP == kColGather;
+  static constexpr bool SCATTER = RTC && LP == kColScatter;
   static constexpr int LOG2NT = LOG2N + LOG2PRE;        // transform length n
   static constexpr int LOG2RPS = LOG2L - LOG2R;   // rows per sub-transform
   static constexpr int LOG2GG = LOG2GPTS - LOG2L; // sub-transforms per item
@@ -181,7 +199,7 @@ struct Geo {
 };
 
 // Rows of a column pass's one-level twiddle table.
-constexpr int kLog2ColRows = 10;
+constexpr int kLog2ColRows = 8;
 
 // Runtime part of a pass.
 struct PRun {
@@ -194,9 +212,8 @@ struct PRun {
   const float2 *tw_stage;         // stage twiddles [t][j][lo]
   unsigned long long swz_tab;     // SMEM swizzle nibble per (ul & 15)
   int last_img;                   // byte offset of the last stage's F images
-  // kSingle: if set, output k of sub-transform u is multiplied by
-  // spec[(u & spec_mask) L + k] (a 2-D spectrum whose rows are the
-  // sub-transforms: the pointwise product of a circular convolution)
+  // the spectrum of a circular convolution: row u & spec_mask of L values
+  // (convolution rows), or one array of outputs (kColSpectrum)
   const float2 *spec;
   long long spec_mask;
   // process the items last to first: set on a pass that reads what the
@@ -208,6 +225,12 @@ struct PRun {
   // the columns n2; its twiddles are tw_out[row of rest][k] (rows beyond
   // kColRows: tw_out[row mod kColRows][k] times tw_b[row / kColRows][k])
   int lo, lp, lc;
+  // real tiles (kColGather, kColScatter, kRealConv): the side x side grid, its
+  // tiles per row, output block side and halo; rows of a half spectrum
+  const float *grid_in;
+  float *grid_out;
+  long long side;
+  int tpr, block, halo, half;
 };
 
 struct GArgs {
@@ -681,8 +704,86 @@ __device__ __forceinline__ void stage_rows(const PRun &P, const WG &w) {
   }
 }
 
+// ---- real tiles.  Column v of a tile's packed array holds the tile's real
+// columns 2 v (real part) and 2 v + 1 (imaginary part); a tile is the window
+// of output block (r, c): grid rows r B - k .., columns c B - k .. (zero outside
+// the grid), N x N points of which the centred B x B are the block's outputs.
+
+// This thread's stage-1 row of `item` from the grid into its own places of the
+// staging buffer (the ones staged_row reads back, so no other thread is
+// involved), asynchronously: 4- or 8-byte copies, as the window's column offset
+// and the grid's row pitch give no alignment a tensor copy could use.  Bound by
+// issue: with the bounds and the alignment tested once a row instead of once
+// a value the pass went from 51 to 38 us (4096^2 in 361 tiles of 256^2).
+template <class G>
+__device__ __forceinline__ void gather_rows(const PRun &P, const WG &w, long long item) {
+  constexpr int R = 1 << G::LOG2R;
+  int ul, q;
+  row_of<G>(G::MODE_FIRST, w.rho, ul, q);
+  constexpr int JS = 1 << (G::LOG2L - G::LOG2R);
+  const long long u = (item << G::LOG2GG) + ul;
+  const unsigned tile = (unsigned)(u >> P.lo);
+  const int v = (int)(u & ((1ll << P.lo) - 1));
+  const unsigned tr = tile / (unsigned)P.tpr, tc = tile - tr * (unsigned)P.tpr;
+  const long long gj = (long long)tc * P.block - P.halo + 2 * v;
+  const long long gi = (long long)tr * P.block - P.halo + q;
+  const long long step = JS * P.side;  // a multiple of 8 floats
+  const float *src = P.grid_in + gi * P.side + gj;
+  const uint32_t dst = smem_u32(w.stg + q * G::GG + ul);
+  if (gi >= 0 && gi + (R - 1) * JS < P.side && gj >= 0 && gj + 1 < P.side &&
+      ((uintptr_t)src & 7) == 0) {
+    // inside the grid, on an 8-byte boundary in every row
+#pragma unroll
+    for (int j = 0; j < R; ++j, src += step) cp_async8(dst + j * (JS * G::GG * 8), src);
+    return;
+  }
+  const bool in0 = gj >= 0 && gj < P.side, in1 = gj + 1 >= 0 && gj + 1 < P.side;
+#pragma unroll 4
+  for (int j = 0; j < R; ++j, src += step) {
+    const bool row = gi + j * JS >= 0 && gi + j * JS < P.side;
+    const uint32_t at = dst + j * (JS * G::GG * 8);
+    cp_async4(at, row && in0 ? src : P.grid_in, row && in0);
+    cp_async4(at + 4, row && in1 ? src + 1 : P.grid_in, row && in1);
+  }
+}
+
+// The outputs k = klow + j r^(S-1) of packed column v (sub-transform u) back to
+// the grid: those inside the tile's output block and the grid.
+template <class G>
+__device__ __forceinline__ void scatter_rows(const PRun &P, const WG &w, long long u, int klow,
+                                             const float *d) {
+  constexpr int R = 1 << G::LOG2R;
+  constexpr int JS = 1 << (G::LOG2L - G::LOG2R);
+  const unsigned tile = (unsigned)(u >> P.lo);
+  const int v = (int)(u & ((1ll << P.lo) - 1));
+  const unsigned tr = tile / (unsigned)P.tpr, tc = tile - tr * (unsigned)P.tpr;
+  const int c0 = 2 * v - P.halo;  // column within the block
+  const long long gj = (long long)tc * P.block + c0;
+  const bool in0 = c0 >= 0 && c0 < P.block && gj < P.side;
+  const bool in1 = c0 + 1 >= 0 && c0 + 1 < P.block && gj + 1 < P.side;
+  if (!in0 && !in1) return;
+  const int r0 = klow - P.halo;  // row of j = 0 within the block
+  const long long i0 = (long long)tr * P.block;
+  const int rows = (int)min((long long)P.block, P.side - i0);
+  const long long step = JS * P.side;
+  float *dst = P.grid_out + (i0 + r0) * P.side + gj;
+  if (in0 && in1 && ((uintptr_t)dst & 7) == 0) {  // on an 8-byte boundary in every row
+#pragma unroll
+    for (int j = 0; j < R; ++j, dst += step)
+      if ((unsigned)(r0 + j * JS) < (unsigned)rows)
+        __stcs(reinterpret_cast<float2 *>(dst), make_float2(d[2 * j], d[2 * j + 1]));
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < R; ++j, dst += step)
+    if ((unsigned)(r0 + j * JS) < (unsigned)rows) {
+      if (in0) __stcs(dst, d[2 * j]);
+      if (in1) __stcs(dst + 1, d[2 * j + 1]);
+    }
+}
+
 // Last stage: D -> registers -> natural-order output.
-template <class G, int PREC, bool OUT_L2, bool SPEC = true>
+template <class G, int PREC, bool OUT_L2>
 __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, WG &w) {
   constexpr int R = 1 << G::LOG2R;
   constexpr int S = G::LOG2L / G::LOG2R;
@@ -704,6 +805,10 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   for (int i = 0; i < S - 1; ++i) {
     klow = (klow << G::LOG2R) | (vq & (R - 1));
     vq >>= G::LOG2R;
+  }
+  if constexpr (G::SCATTER) {
+    scatter_rows<G>(P, w, u, klow, d);
+    return;
   }
   long long b = u >> log2_uper<G>(P);
   long long v = u & ((1ll << log2_uper<G>(P)) - 1);
@@ -747,9 +852,8 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   const float2 *twbs = w.twb + klow;
   const float2 *twbg = P.tw_b + (vh << G::LOG2L) + klow;
   constexpr int TBJ = 1 << (G::LOG2L - G::LOG2R);
-  const long long soff = ((u & P.spec_mask) << G::LOG2L) + klow;
-  const float2 *sp = P.spec + soff;
-  const bool mul = SPEC && G::MODE_LAST == kRQF && P.spec != nullptr;
+  // kColSpectrum: the spectrum entry of output e of the array is spec[e]
+  const float2 *sp = P.spec + (dst - P.out) - (G::RTC ? (b >> P.lp) << (P.lo + P.lp + G::LOG2L) : 0);
   // index bounds of the checked build (element offsets from each base)
   const long long doff = dst - P.out;
   const long long out_elems =
@@ -760,16 +864,17 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   // The factors of a chunk of outputs (spectrum, twiddles) are loaded before
   // its stores: the stores are asm with a memory clobber, so a load written
   // after one of them would wait for it, a round trip per value.
-  constexpr int CH = (G::TW2L || G::MODE_LAST == kRQF) ? 8 : load_chunk(R, G::NWG);
+  constexpr int CH = G::TW2L ? 8 : load_chunk(R, G::NWG);
 #pragma unroll
   for (int c = 0; c < R; c += CH) {
-    float2 fs[CH], fa[CH], fb[CH];
+    float2 fa[CH], fb[CH];
 #pragma unroll
     for (int jj = 0; jj < CH; ++jj) {
       const int j = c + jj;
-      if (G::MODE_LAST == kRQF && mul)
-        fs[jj] = in_range(w, soff + j * JS, (P.spec_mask + 1) << G::LOG2L) ? __ldg(sp + j * JS)
-                                                                          : one;
+      if (G::RTC_SPEC)
+        fa[jj] = in_range(w, (sp - P.spec) + j * JS, 1ll << (P.lo + P.lp + G::LOG2L))
+                     ? __ldg(sp + j * JS)
+                     : one;
       if (G::RTC_TW) {
         fa[jj] = in_range(w, coff + j * TBJ, c_elems) ? __ldg(P.tw_out + coff + j * TBJ) : one;
         if (ctwo && in_range(w, cboff + j * TBJ, cb_elems))
@@ -791,8 +896,7 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
     for (int jj = 0; jj < CH; ++jj) {
       const int j = c + jj;
       float2 y = make_float2(d[2 * j], d[2 * j + 1]);
-      if (G::MODE_LAST == kRQF && mul) y = cmul(y, fs[jj]);
-      if (G::RTC_TW) y = cmul(y, fa[jj]);
+      if (G::RTC_TW || G::RTC_SPEC) y = cmul(y, fa[jj]);
       if (G::TW_SMEM || G::TW_OUT) y = G::TW2L ? cmul(y, cmul(fa[jj], fb[jj])) : cmul(y, fa[jj]);
       if (in_range(w, doff + j * JS, out_elems)) {
         if (OUT_L2)
@@ -813,8 +917,12 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
                                              Mid &mid) {
   constexpr int R = 1 << G::LOG2R;
   constexpr int S = G::LOG2L / G::LOG2R;
-  if (!mbar_wait_bounded(w.bar_stg, w.ph_stg)) w.fail = true;
-  w.ph_stg ^= 1;
+  if constexpr (G::GATHER) {
+    cp_async_wait_all();  // this thread's own copies
+  } else {
+    if (!mbar_wait_bounded(w.bar_stg, w.ph_stg)) w.fail = true;
+    w.ph_stg ^= 1;
+  }
   mid.after_load(w);
   {
     float2 x[R];
@@ -824,6 +932,8 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
       split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
                          w.slot + G::Q + w.lane_off + a_cols8(PREC) * c / 8);
   }
+  // the row is in TMEM: this thread's places of the staging are free again
+  if constexpr (G::GATHER) mid.issue(w);
   tmem_wait_st();
   fence_before_sync();
   if (named_bar_or(w.bar_id, w.bar_count, w.fail)) {
@@ -840,7 +950,7 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
       issue_twiddles<G>(P, tm_tw, item, w);
       w.tws_inflight = true;
     }
-    mid.issue(w);
+    if constexpr (!G::GATHER) mid.issue(w);
   }
   if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
   w.ph_mma ^= 1;
@@ -953,8 +1063,13 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
   constexpr int R = 1 << G::LOG2R, H = R / 2;
   constexpr int S = G::LOG2L / G::LOG2R;
   static_assert(G::KS && S <= 2 && !G::TW_SMEM, "half-K items: radix 32, at most two stages");
-  if (!mbar_wait_bounded(w.bar_stg, w.ph_stg)) w.fail = true;
-  w.ph_stg ^= 1;
+  static_assert(!G::GATHER || S == 2, "gathered columns are whole warpgroup passes");
+  if constexpr (G::GATHER) {
+    cp_async_wait_all();  // this thread's own copies
+  } else {
+    if (!mbar_wait_bounded(w.bar_stg, w.ph_stg)) w.fail = true;
+    w.ph_stg ^= 1;
+  }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     {
@@ -1001,7 +1116,7 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
         issue_stage_half<R, PREC, G::QA>(h, w.slot, w.img_addr + P.last_img, w.bar_mma);
       }
       // the transpose buffer (shared with the staging) has been read
-      if (h == 1 && w.team_lead) mid.issue(w);
+      if (h == 1 && (G::GATHER || w.team_lead)) mid.issue(w);
       if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
       w.ph_mma ^= 1;
       fence_after_sync();
@@ -1020,7 +1135,7 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
 // map, same TMEM lane): it multiplies them by the spectrum and stores them
 // straight back as its A operand.  F images in SMEM: forward hi, lo at 0,
 // inverse hi, lo at 2 IMG; stage twiddles tw_f (forward), tw_i (inverse).
-template <class G, int PREC>
+template <class G, int PREC, int CONV>
 __device__ __forceinline__ void conv_turn(const PRun &P, long long item, const WG &w) {
   constexpr int R = 1 << G::LOG2R;
   constexpr int S = G::LOG2L / G::LOG2R;
@@ -1035,7 +1150,10 @@ __device__ __forceinline__ void conv_turn(const PRun &P, long long item, const W
   const long long u = (item << G::LOG2GG) + ul;
   float d[2 * R];
   load_d_row<G, PREC>(w, d);
-  const float2 *sp = P.spec + ((u & P.spec_mask) << G::LOG2L) + klow;
+  // the spectrum's row: of a half spectrum u modulo its rows
+  const long long srow =
+      CONV == kRealConv ? (unsigned)u % (unsigned)P.half : u & P.spec_mask;
+  const float2 *sp = P.spec + (srow << G::LOG2L) + klow;
   constexpr int JS = 1 << (G::LOG2L - G::LOG2R);
 #pragma unroll
   for (int c = 0; c < R; c += 8) {
@@ -1043,7 +1161,8 @@ __device__ __forceinline__ void conv_turn(const PRun &P, long long item, const W
 #pragma unroll
     for (int jj = 0; jj < 8; ++jj) {
 #ifdef TCU_DFT_CHECKED
-      const float2 s = in_range(w, (sp - P.spec) + (c + jj) * JS, (P.spec_mask + 1) << G::LOG2L)
+      const float2 s = in_range(w, (sp - P.spec) + (c + jj) * JS,
+                                (CONV == kRealConv ? P.half : P.spec_mask + 1) << G::LOG2L)
                            ? __ldg(sp + (c + jj) * JS)
                            : make_float2(0.f, 0.f);
 #else
@@ -1053,6 +1172,102 @@ __device__ __forceinline__ void conv_turn(const PRun &P, long long item, const W
     }
     split_store8<PREC>(x, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
                        w.slot + G::Q + w.lane_off + a_cols8(PREC) * c / 8);
+  }
+}
+
+// ---- rows of real tiles.  The column transforms Z of a packed tile (N rows of
+// N / 2 values, Z = X_even + i X_odd for the spectra X of its real columns)
+// determine the rows k1 = 0 .. N / 2 of the tile's column spectra, X[N - k1]
+// being conj X[k1]: sub-transform u = tile half + k1 (half = N / 2 + 1) is row k1
+// of N values, untangled from the rows k1 and N - k1 of Z as it is read, and
+// packed again into the same two rows as it is stored, so the pass runs in
+// place on half the rows a complex tile has.
+
+// The two rows of Z of every sub-transform of `item` into staging [ul][Z k1 |
+// Z (N - k1)]: one copy per lane (a warp, converged).
+template <class G>
+__device__ __forceinline__ void issue_half_rows(const PRun &P, long long item, const WG &w) {
+  constexpr int HALF = G::L / 2;
+  static_assert(2 * G::GG <= 32, "a lane per copy");
+  const int lane = threadIdx.x & 31;
+  const long long u0 = item << G::LOG2GG;
+  long long rem = P.U - u0;
+  if (rem > G::GG) rem = G::GG;
+  const long long u = u0 + (lane >> 1);
+  const long long tile = (unsigned)u / (unsigned)P.half;
+  const int k1 = (int)(u - tile * P.half), row = lane & 1 ? (G::L - k1) & (G::L - 1) : k1;
+  const long long off = (tile << (2 * G::LOG2L - 1)) + (long long)row * HALF;
+  const bool mine = (lane >> 1) < rem;
+  const bool ok = !mine || in_range(w, off + HALF - 1, (P.U / P.half) << (2 * G::LOG2L - 1));
+  const bool all = __all_sync(0xffffffffu, ok);
+  if (lane == 0) mbar_expect_tx(w.bar_stg, all ? (uint32_t)(rem * G::L * 8) : 0u);
+  __syncwarp();
+  if (all && mine)
+    tma_load_1d(smem_u32(w.stg) + lane * (HALF * 8), P.in + off, HALF * 8, w.bar_stg);
+  __syncwarp();
+}
+
+// This thread's stage-1 row: value c = 2 v or 2 v + 1 of row k1 is
+// (Z + conj Z') / 2 or (Z - conj Z') / 2i, Z = Z[k1][v], Z' = Z[N - k1][v].
+template <class G>
+__device__ __forceinline__ void staged_half_row(const WG &w, float2 *x) {
+  constexpr int R = 1 << G::LOG2R;
+  constexpr int JS = 1 << (G::LOG2L - G::LOG2R);  // c = j * R^(S-1) + q
+  constexpr int HALF = G::L / 2;
+  static_assert(JS % 2 == 0 || G::LOG2L == G::LOG2R, "one parity per row");
+  int ul, q;
+  row_of<G>(kQF, w.rho, ul, q);
+  const int i0 = (ul << G::LOG2L) + (q >> 1);
+  const bool odd = q & 1;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int i = i0 + j * (JS / 2);
+    const float2 zero = make_float2(0.f, 0.f);
+    const float2 z = in_range(w, i, G::GPTS) ? w.stg[i] : zero;
+    const float2 y = in_range(w, i + HALF, G::GPTS) ? w.stg[i + HALF] : zero;
+    const float sr = z.x + y.x, si = z.y - y.y;  // Z + conj Z'
+    const float dr = z.x - y.x, di = z.y + y.y;  // Z - conj Z'
+    x[j] = odd ? make_float2(0.5f * di, -0.5f * dr) : make_float2(0.5f * sr, 0.5f * si);
+  }
+}
+
+// The last inverse stage of a row: lanes 2 i, 2 i + 1 hold the columns 2 v and
+// 2 v + 1; together they form Z[k1][v] = Ye + i Yo (stored by the even lane) and
+// Z[N - k1][v] = conj Ye + i conj Yo (the odd lane).  Rows 0 and N / 2 are their
+// own partners; their column spectra are real, and Z is Re Ye + i Re Yo.
+template <class G, int PREC>
+__device__ __forceinline__ void half_row_store(const PRun &P, long long item, WG &w) {
+  constexpr int R = 1 << G::LOG2R;
+  constexpr int S = G::LOG2L / G::LOG2R;
+  int ul, q;
+  row_of<G>(kRQF, w.rho, ul, q);
+  const long long u = (item << G::LOG2GG) + ul;
+  float d[2 * R];
+  load_d_row<G, PREC>(w, d);
+  int klow = 0, vq = q;
+#pragma unroll
+  for (int i = 0; i < S - 1; ++i) {
+    klow = (klow << G::LOG2R) | (vq & (R - 1));
+    vq >>= G::LOG2R;
+  }
+  const long long tile = (unsigned)u / (unsigned)P.half;
+  const int k1 = (int)(u - tile * P.half);
+  const bool odd = klow & 1, self = k1 == 0 || k1 == G::L / 2;
+  const int row = odd ? G::L - k1 : k1;
+  const long long off =
+      (tile << (2 * G::LOG2L - 1)) + (long long)row * (G::L / 2) + (klow >> 1);
+  const bool store = u < P.U && !(odd && self);
+  constexpr int JS = 1 << (G::LOG2L - G::LOG2R);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const float px = __shfl_xor_sync(0xffffffffu, d[2 * j], 1);
+    const float py = __shfl_xor_sync(0xffffffffu, d[2 * j + 1], 1);
+    // even: (Ye.x - Yo.y, Ye.y + Yo.x); odd: (Ye.x + Yo.y, Yo.x - Ye.y)
+    float2 z = odd ? make_float2(px + d[2 * j + 1], d[2 * j] - py)
+                   : make_float2(d[2 * j] - py, d[2 * j + 1] + px);
+    if (self) z = make_float2(d[2 * j], px);
+    if (store && in_range(w, off + j * (JS / 2), (P.U / P.half) << (2 * G::LOG2L - 1)))
+      __stcg(P.out + off + j * (JS / 2), z);
   }
 }
 
@@ -1090,7 +1305,7 @@ __device__ __forceinline__ bool later_stages(const PRun &P, const float2 *tws, W
   return true;
 }
 
-template <class G, int PREC, class Mid>
+template <class G, int PREC, int CONV, class Mid>
 __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *tw_f,
                                                   const float2 *tw_i, long long item, WG &w,
                                                   Mid &mid) {
@@ -1100,7 +1315,10 @@ __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *t
   w.ph_stg ^= 1;
   {
     float2 x[R];
-    staged_row<G>(w, x);
+    if constexpr (CONV == kRealConv)
+      staged_half_row<G>(w, x);
+    else
+      staged_row<G>(w, x);
 #pragma unroll
     for (int c = 0; c < R; c += 8)
       split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
@@ -1122,7 +1340,7 @@ __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *t
   fence_after_sync();
   if (!later_stages<G, PREC>(P, tw_f, w, 0, mid, true)) return;
   // the turn: forward outputs times the spectrum become the inverse A rows
-  conv_turn<G, PREC>(P, item, w);
+  conv_turn<G, PREC, CONV>(P, item, w);
   tmem_wait_st();
   fence_before_sync();
   if (named_bar_or(w.bar_id, w.bar_count, w.fail)) {
@@ -1137,7 +1355,10 @@ __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *t
   w.ph_mma ^= 1;
   fence_after_sync();
   if (!later_stages<G, PREC>(P, tw_i, w, INV, mid, false)) return;
-  last_stage_store<G, PREC, false, false>(P, item, w);
+  if constexpr (CONV == kRealConv)
+    half_row_store<G, PREC>(P, item, w);
+  else
+    last_stage_store<G, PREC, false>(P, item, w);
 }
 
 // Common set-up: mbarriers, TMEM, and the F images and stage twiddles into
@@ -1246,22 +1467,30 @@ __device__ __forceinline__ void init_wg(WG &w, uint32_t tbase, unsigned char *sm
 }
 
 // ---------------------------------------------------------------- one pass
-template <class G>
+template <class G, int CONV>
 struct StaticNext {
   const PRun &P;
   const CUtensorMap *tm;
   long long next, nitems;
   bool issued;  // a copy for `next` is in flight
+  // one warp, converged -- or, for gathered columns, every thread
   __device__ void issue(const WG &w) {
     issued = next < nitems;
-    if (issued) issue_input<G>(P, tm, G::TW == 1 && P.reverse ? nitems - 1 - next : next, w);
+    if (!issued) return;
+    const long long at = G::TW == 1 && P.reverse ? nitems - 1 - next : next;
+    if constexpr (G::GATHER)
+      gather_rows<G>(P, w, at);
+    else if constexpr (CONV == kRealConv)
+      issue_half_rows<G>(P, at, w);
+    else
+      issue_input<G>(P, tm, at, w);
   }
   __device__ void publish() {}
   __device__ void after_load(const WG &) {}
   __device__ void before_store(WG &) {}
 };
 
-template <int R, int PREC, int S, int LO, int ROLE, int LP, bool CONV = false, int TW = 1>
+template <int R, int PREC, int S, int LO, int ROLE, int LP, int CONV = kNoConv, int TW = 1>
 __global__ void __launch_bounds__(
     Geo<R, S, LO, ROLE, LP,
         TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>::THREADS,
@@ -1300,22 +1529,23 @@ __global__ void __launch_bounds__(
   const long long istride = (long long)gridDim.x * G::NTEAM;
   // team-major: with fewer items than SMs each CTA holds one item
   long long item = (long long)team * gridDim.x + blockIdx.x;
-  StaticNext<G> nx{P, &a.tm_in, item, nitems, false};
+  StaticNext<G, CONV> nx{P, &a.tm_in, item, nitems, false};
   // item: position in this CTA's sequence; phys: the item processed there
   // (team passes always run forward: no reversal code in them)
   auto phys = [&](long long i) { return TW == 1 && P.reverse ? nitems - 1 - i : i; };
   // the first input copy of team 0 leaves with the tables (warp 0 set up its
   // mbarriers), the other teams' after the CTA barrier
-  if (team == 0 && w.team_lead && item < nitems) issue_input<G>(P, &a.tm_in, phys(item), w);
+  // (gathered columns: every thread copies its own row, after the barrier)
+  if (!G::GATHER && team == 0 && w.team_lead) nx.issue(w);
   const uint32_t tbase = kernel_setup_finish(tmem_slot);
   w.slot = tbase + (uint32_t)((threadIdx.x >> 7) * G::GCOLS);
-  if (team != 0 && w.team_lead && item < nitems) issue_input<G>(P, &a.tm_in, phys(item), w);
+  if (G::GATHER || (team != 0 && w.team_lead)) nx.issue(w);
   // the tables have landed (the same answer in every thread of the team)
   if (named_bar_or(w.bar_id, w.bar_count, !wait_tables(mbar, G::NWG))) w.fail = true;
   while (item < nitems && !w.fail) {
     nx.next = item + istride;
-    if constexpr (CONV)
-      process_item_conv<G, PREC>(P, tw, tw_inv, phys(item), w, nx);
+    if constexpr (CONV != kNoConv)
+      process_item_conv<G, PREC, CONV>(P, tw, tw_inv, phys(item), w, nx);
     else if constexpr (G::KS)
       process_item_ks<G, PREC>(P, tw, phys(item), w, nx);
     else
@@ -1327,7 +1557,8 @@ __global__ void __launch_bounds__(
   }
   if (w.fail && w.rho == 0) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);
   // on failure a copy issued for the next item may still be landing
-  kernel_teardown(tbase, w, w.fail && nx.issued, w.fail && w.tws_inflight);
+  if (G::GATHER) cp_async_wait_all();
+  kernel_teardown(tbase, w, !G::GATHER && w.fail && nx.issued, w.fail && w.tws_inflight);
 }
 
 // ------------------------------------------------------- fused two passes

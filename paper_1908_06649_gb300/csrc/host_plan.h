@@ -200,6 +200,9 @@ void free_plan(tcu_dft_plan_s *p);
 // ---------------------------------------------------------------- launches
 cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, int num_sms,
                           cudaStream_t st);
+// A column pass of a 2-D transform (mode: ColMode).
+cudaError_t launch_cols(int r, int prec, int s, int mode, const GArgs &a, int num_sms,
+                        cudaStream_t st);
 cudaError_t fused_dispatch(int r, int prec, int s1, int s2, const GArgs &a, int num_sms,
                            cudaStream_t st);
 // Warpgroup-kernel description of pass `pi` between buffers `in` and `out`.
@@ -210,13 +213,10 @@ void dir_tables(const tcu_dft_plan_s *p, int d, DirTables &t);
 // The transform of transforms [b0, b0 + count) of the plan's batch (in and
 // out point at transform b0; count < 0: the whole batch).  The intermediates
 // of that range sit at the same offset in the plan's scratch, so disjoint
-// ranges may run concurrently on different streams (not fused plans).  spec:
-// for a plan of one pass, transform b is multiplied by the spectrum row
-// spec[(b & spec_mask) n ...] as it is stored (the rows of a 2-D convolution).
+// ranges may run concurrently on different streams (not fused plans).
 int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
                      void *stream, void *const *events, long long queue_start = 0,
-                     long long b0 = 0, long long count = -1, const float2 *spec = nullptr,
-                     long long spec_mask = 0);
+                     long long b0 = 0, long long count = -1);
 
 }  // namespace host
 }  // namespace tcu

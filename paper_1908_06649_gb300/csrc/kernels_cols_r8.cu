@@ -4,16 +4,25 @@
 
 namespace tcu {
 
-// (stages, with an inter-pass twiddle)
-cudaError_t launch_cols_r8(int prec, int s, int twid, const GArgs &a, int num_sms,
+// (stages, ColMode)
+cudaError_t launch_cols_r8(int prec, int s, int mode, const GArgs &a, int num_sms,
                            cudaStream_t st) {
   constexpr int R = 8;
-  TCU_COLS_CASE(1, 0, launch_pass_t)
-  TCU_COLS_CASE(2, 0, launch_pass_t)
-  TCU_COLS_CASE(3, 0, launch_team_t, TCU_COMMA 4)
-  TCU_COLS_CASE(1, 1, launch_pass_t)
-  TCU_COLS_CASE(2, 1, launch_pass_t)
-  TCU_COLS_CASE(3, 1, launch_team_t, TCU_COMMA 4)
+  TCU_COLS_CASE(1, kColPlain)
+  TCU_COLS_CASE(2, kColPlain)
+  TCU_COLS_TEAM_CASE(3, kColPlain, 4)
+  TCU_COLS_CASE(1, kColTwiddle)
+  TCU_COLS_CASE(2, kColTwiddle)
+  TCU_COLS_TEAM_CASE(3, kColTwiddle, 4)
+  TCU_COLS_CASE(1, kColSpectrum)
+  TCU_COLS_CASE(2, kColSpectrum)
+  TCU_COLS_TEAM_CASE(3, kColSpectrum, 4)
+  if (prec != 3) return cudaErrorInvalidValue;
+  // real tiles: 64 and 512 points a side
+  if (s == 2 && mode == kColGather) return launch_pass_t<R, 3, 2, 0, kCols, kColGather>(a, num_sms, st);
+  if (s == 2 && mode == kColScatter) return launch_pass_t<R, 3, 2, 0, kCols, kColScatter>(a, num_sms, st);
+  if (s == 3 && mode == kColGather) return launch_team_t<R, 3, 3, 0, kCols, kColGather, 4>(a, num_sms, st);
+  if (s == 3 && mode == kColScatter) return launch_team_t<R, 3, 3, 0, kCols, kColScatter, 4>(a, num_sms, st);
   return cudaErrorInvalidValue;
 }
 

@@ -35,11 +35,12 @@ cudaError_t launch_pair_r16(int prec, int s1, int s2, const GArgs &a, int cluste
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_rowconv_r16(int prec, int s, const GArgs &a, int num_sms,
+cudaError_t launch_rowconv_r16(int prec, int s, bool real, const GArgs &a, int num_sms,
                                cudaStream_t st) {
   constexpr int R = 16;
   TCU_ROWCONV_CASE(1)
   TCU_ROWCONV_CASE(2)
+  TCU_REAL_ROWCONV_CASE(2)
   return cudaErrorInvalidValue;
 }
 

@@ -29,11 +29,12 @@ cudaError_t launch_fused_r32(int prec, int s1, int s2, const GArgs &a, int num_s
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_rowconv_r32(int prec, int s, const GArgs &a, int num_sms,
+cudaError_t launch_rowconv_r32(int prec, int s, bool real, const GArgs &a, int num_sms,
                                cudaStream_t st) {
   constexpr int R = 32;
   TCU_ROWCONV_CASE(1)
   TCU_ROWCONV_CASE(2)
+  TCU_REAL_ROWCONV_CASE(2)
   return cudaErrorInvalidValue;
 }
 

@@ -17,20 +17,23 @@ cudaError_t launch_pass_r16(int prec, int s, int lo, int role, int lp, const GAr
                             int num_sms, cudaStream_t st);
 cudaError_t launch_pass_r32(int prec, int s, int lo, int role, int lp, const GArgs &a,
                             int num_sms, cudaStream_t st);
-// A column pass of a 2-D transform whose columns need several passes, or of a
-// BF16 mode (kernels_cols_r*.cu): s stages, twid: with the inter-pass twiddle;
-// the shape is in a.p[0].lo, lp, lc.
-cudaError_t launch_cols_r8(int prec, int s, int twid, const GArgs &a, int num_sms,
+// A column pass of a 2-D transform (kernels_cols_r*.cu): s stages, mode a
+// ColMode; the shape is in a.p[0].lo, lp, lc.
+cudaError_t launch_cols_r8(int prec, int s, int mode, const GArgs &a, int num_sms,
                            cudaStream_t st);
-cudaError_t launch_cols_r16(int prec, int s, int twid, const GArgs &a, int num_sms,
+cudaError_t launch_cols_r16(int prec, int s, int mode, const GArgs &a, int num_sms,
                             cudaStream_t st);
-cudaError_t launch_cols_r32(int prec, int s, int twid, const GArgs &a, int num_sms,
+cudaError_t launch_cols_r32(int prec, int s, int mode, const GArgs &a, int num_sms,
                             cudaStream_t st);
 // The row pass of a circular 2-D convolution: each row transformed,
-// multiplied by the spectrum and transformed back on chip (s stages).
-cudaError_t launch_rowconv_r8(int prec, int s, const GArgs &a, int num_sms, cudaStream_t st);
-cudaError_t launch_rowconv_r16(int prec, int s, const GArgs &a, int num_sms, cudaStream_t st);
-cudaError_t launch_rowconv_r32(int prec, int s, const GArgs &a, int num_sms, cudaStream_t st);
+// multiplied by the spectrum and transformed back on chip (s stages); real:
+// of packed real tiles.
+cudaError_t launch_rowconv_r8(int prec, int s, bool real, const GArgs &a, int num_sms,
+                              cudaStream_t st);
+cudaError_t launch_rowconv_r16(int prec, int s, bool real, const GArgs &a, int num_sms,
+                               cudaStream_t st);
+cudaError_t launch_rowconv_r32(int prec, int s, bool real, const GArgs &a, int num_sms,
+                               cudaStream_t st);
 // Both passes of a two-pass transform in one launch on clusters of two CTAs,
 // each cluster's intermediate in two L2-resident slots (radix 16, 2 + 2).
 cudaError_t launch_pair_r16(int prec, int s1, int s2, const GArgs &a, int clusters,
@@ -50,6 +53,9 @@ struct Stencil3 {
 cudaError_t launch_place_poly(float2 *g, long long Nw, const Stencil3 &w, int num_sms,
                               cudaStream_t st);
 cudaError_t launch_cpow(float2 *g, long long count, int k, int num_sms, cudaStream_t st);
+// Rows 0 .. N / 2 of the spectrum of the kernel of k steps (roots: w_N^{-f}).
+cudaError_t launch_stencil_spectrum(float2 *S, const double2 *roots, long long N,
+                                    const Stencil3 &w, int k, int num_sms, cudaStream_t st);
 cudaError_t launch_extract_weights(float *W, const float2 *g, long long Nw, int k,
                                    int num_sms, cudaStream_t st);
 cudaError_t launch_place_kernel(float2 *w, long long N, const float2 *g, long long Nw, int k,

@@ -30,13 +30,13 @@ template <int R, int PREC, int S, int LO, int ROLE, int LP, int TW>
 cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, LO, ROLE, LP, team_nwg(R), TW>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, 0, G::TW_SMEM, G::TWB, TW>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, false, TW>,
+  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   const long long nitems = (a.p[0].U + G::GG - 1) >> G::LOG2GG;
   long long grid = nitems < num_sms ? nitems : num_sms;
-  dft_pass_kernel<R, PREC, S, LO, ROLE, LP, false, TW>
+  dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>
       <<<(unsigned)grid, G::THREADS, sm, st>>>(a);
   return cudaGetLastError();
 }
@@ -49,24 +49,27 @@ cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   TCU_TEAM_CASE_L(S, log2_radix(R) * (SO), ROLE, log2_radix(R) * (SP), TW)
 
 // The convolution row pass (forward rows, spectrum product, inverse rows).
-template <int R, int PREC, int S>
+template <int R, int PREC, int S, int CONV>
 cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, kSingle, S)>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::TW_ENTRIES, false, 0>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, true>,
+  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   const long long nitems = (a.p[0].U + G::GG - 1) >> G::LOG2GG;
   long long grid = nitems < num_sms ? nitems : num_sms;
-  dft_pass_kernel<R, PREC, S, 0, kSingle, 0, true><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
+  dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
   return cudaGetLastError();
 }
 
 #define TCU_ROWCONV_CASE(S)                                                         \
-  if (s == S)                                                                       \
-    return prec == 3 ? launch_rowconv_t<R, 3, S>(a, num_sms, st)                    \
-                     : launch_rowconv_t<R, 1, S>(a, num_sms, st);
+  if (s == S && !real)                                                              \
+    return prec == 3 ? launch_rowconv_t<R, 3, S, kConv>(a, num_sms, st)             \
+                     : launch_rowconv_t<R, 1, S, kConv>(a, num_sms, st);
+// ... of real tiles (3xTF32)
+#define TCU_REAL_ROWCONV_CASE(S) \
+  if (s == S && real && prec == 3) return launch_rowconv_t<R, 3, S, kRealConv>(a, num_sms, st);
 
 template <int R, int PREC, int S1, int S2>
 cudaError_t launch_fused_t(const GArgs &a, int num_sms, cudaStream_t st) {
@@ -140,16 +143,22 @@ cudaError_t launch_pair_t(const GArgs &a, int clusters, cudaStream_t st) {
                                      log2_radix(R) * (SP), TW>(a, num_sms, st)          \
                      : launch_team_t<R, 4, S, log2_radix(R) * (SO), ROLE,               \
                                      log2_radix(R) * (SP), TW>(a, num_sms, st);
-// A column pass of a 2-D transform (kCols) of S stages, with (TWID = 1) or
-// without its inter-pass twiddle, items of TW warpgroups; every precision.
-#define TCU_COLS_CASE(S, TWID, LAUNCH, ...)                                              \
-  if (s == S && twid == TWID) {                                                          \
-    if (prec == 3) return LAUNCH<R, 3, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
-    if (prec == 1) return LAUNCH<R, 1, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
-    if (prec == 5) return LAUNCH<R, 5, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);  \
-    return LAUNCH<R, 4, S, 0, kCols, TWID __VA_ARGS__>(a, num_sms, st);                 \
+// A column pass of a 2-D transform (kCols) of S stages in ColMode MODE, items
+// of one warpgroup (or, TCU_COLS_TEAM_CASE, of TW); every precision.
+#define TCU_COLS_CASE(S, MODE)                                                            \
+  if (s == S && mode == MODE) {                                                           \
+    if (prec == 3) return launch_pass_t<R, 3, S, 0, kCols, MODE>(a, num_sms, st);         \
+    if (prec == 1) return launch_pass_t<R, 1, S, 0, kCols, MODE>(a, num_sms, st);         \
+    if (prec == 5) return launch_pass_t<R, 5, S, 0, kCols, MODE>(a, num_sms, st);         \
+    return launch_pass_t<R, 4, S, 0, kCols, MODE>(a, num_sms, st);                        \
   }
-#define TCU_COMMA ,
+#define TCU_COLS_TEAM_CASE(S, MODE, TW)                                                   \
+  if (s == S && mode == MODE) {                                                           \
+    if (prec == 3) return launch_team_t<R, 3, S, 0, kCols, MODE, TW>(a, num_sms, st);     \
+    if (prec == 1) return launch_team_t<R, 1, S, 0, kCols, MODE, TW>(a, num_sms, st);     \
+    if (prec == 5) return launch_team_t<R, 5, S, 0, kCols, MODE, TW>(a, num_sms, st);     \
+    return launch_team_t<R, 4, S, 0, kCols, MODE, TW>(a, num_sms, st);                    \
+  }
 #define TCU_FUSED_CASE(S1, S2)                                                      \
   if (s1 == S1 && s2 == S2)                                                         \
     return prec == 3 ? launch_fused_t<R, 3, S1, S2>(a, num_sms, st)                 \

@@ -318,6 +318,21 @@ __device__ __forceinline__ void tma_load_3d(uint32_t smem_dst, const void *tmap,
       : "memory");
 }
 
+// Asynchronous 4- and 8-byte copies global -> shared of this thread (`take`
+// false: zeros are written and nothing is read), and the wait for all of
+// them.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool take) {
+  asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 4, %2;" ::"r"(dst), "l"(src),
+               "r"(take ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ------------------------------------------------------- thread-block clusters
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;

@@ -257,12 +257,6 @@ void free_plan(tcu_dft_plan_s *p) {
 // ---------------------------------------------------------------- launches
 cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, int num_sms,
                           cudaStream_t st) {
-  if (pp.role == kCols) {
-    const int twid = pp.last ? 0 : 1;
-    if (r == 8) return launch_cols_r8(prec, pp.s, twid, a, num_sms, st);
-    if (r == 16) return launch_cols_r16(prec, pp.s, twid, a, num_sms, st);
-    return launch_cols_r32(prec, pp.s, twid, a, num_sms, st);
-  }
   if (pp.mixed) {
     if (r == 8) return launch_pass_mixed_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
     if (r == 16) return launch_pass_mixed_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
@@ -277,6 +271,13 @@ cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, i
   if (r == 8) return launch_pass_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   if (r == 16) return launch_pass_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
   return launch_pass_r32(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
+}
+
+cudaError_t launch_cols(int r, int prec, int s, int mode, const GArgs &a, int num_sms,
+                        cudaStream_t st) {
+  if (r == 8) return launch_cols_r8(prec, s, mode, a, num_sms, st);
+  if (r == 16) return launch_cols_r16(prec, s, mode, a, num_sms, st);
+  return launch_cols_r32(prec, s, mode, a, num_sms, st);
 }
 
 cudaError_t fused_dispatch(int r, int prec, int s1, int s2, const GArgs &a, int num_sms,
@@ -325,8 +326,7 @@ void dir_tables(const tcu_dft_plan_s *p, int d, DirTables &t) {
 
 int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
                      void *stream, void *const *events, long long queue_start,
-                     long long b0, long long count, const float2 *spec,
-                     long long spec_mask) {
+                     long long b0, long long count) {
   if (!p || !in || !out || (dir != TCU_DFT_FORWARD && dir != TCU_DFT_INVERSE))
     return TCU_DFT_ERR_INVALID;
   if (((uintptr_t)in & 15) || ((uintptr_t)out & 15)) return TCU_DFT_ERR_INVALID;
@@ -427,8 +427,6 @@ int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
       if (!input_map(&g.tm_in, src, p, pp, count)) return TCU_DFT_ERR_CUDA;
       g.tm_tw = pp.tw_map[di];
     }
-    g.p[0].spec = spec;
-    g.p[0].spec_mask = spec_mask;
     g.bimg = p->bimg[di];
     g.err = p->err;
     if (pass_dispatch(p->r, p->precision, pp, g, p->num_sms, st) != cudaSuccess)

@@ -94,3 +94,30 @@ def test_column_passes_conv(pkg, r, n1, n2, batch, prec):
     err = np.linalg.norm(y.cpu().numpy().reshape(batch, -1) - ref, axis=1)
     assert (err / np.linalg.norm(ref, axis=1)).max() <= 2 * TOL[prec]
     plan.destroy()
+
+
+# real tiles (3xTF32): every radix and tile size, the smallest grids (less than
+# a tile), cut blocks, odd sides (rows on no 8-byte boundary), one step, the
+# last step count whose spectrum is evaluated directly and the one after it;
+# weights without any symmetry.  Bar: 1e-5 max |A|, the stencil tests' bar (the
+# weights have unit sum and are not negative).
+@pytest.mark.parametrize("r,side,k", [
+    (8, 1, 1), (8, 37, 5), (8, 129, 21), (8, 600, 24), (8, 460, 25), (16, 1, 1), (16, 225, 1),
+    (16, 449, 16), (16, 448, 16), (16, 300, 24), (16, 301, 25), (16, 500, 85), (32, 33, 2),
+    (32, 1000, 24), (32, 1025, 40)])
+def test_real_tiles(pkg, r, side, k):
+    import torch
+    rng = np.random.default_rng(100 * side + k)
+    A = rng.standard_normal((side, side)).astype(np.float32)
+    w3 = rng.uniform(0.05, 1.0, (3, 3))
+    w3 = (w3 / w3.sum()).astype(np.float32)
+    plan = pkg.StencilPlan(side, k, r, 3)
+    Ad = torch.from_numpy(A).cuda()
+    got = plan.apply(Ad, w3x3=w3.tolist())
+    plan.check()
+    ref = grid.stencil_direct(A.astype(np.float64), w3.astype(np.float64), k)
+    assert np.max(np.abs(got.cpu().numpy() - ref)) <= 1e-5 * np.max(np.abs(A))
+    plan.apply(Ad, Ad, w3x3=w3.tolist())  # in place
+    plan.check()
+    assert torch.equal(Ad, got)
+    plan.destroy()
