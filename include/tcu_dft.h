@@ -148,7 +148,10 @@ int tcu_dft_exec_dir(tcu_dft_plan_t p, const void *in, void *out, int dir,
 /* Same as tcu_dft_exec_dir, and records `events[i]` (cudaEvent_t handles,
  * caller-created) on `stream` just before pass i and events[npasses] after
  * the last pass, so the caller can time each pass kernel on the stream it
- * runs on.  `events` must hold tcu_dft_num_passes(p) + 1 entries. */
+ * runs on.  `events` must hold tcu_dft_num_passes(p) + 1 entries.  Passes that
+ * share a launch (the q-point pass of a mixed-radix n where it rides on the
+ * next, a fused schedule) are timed with one of them; the other's span is
+ * empty. */
 int tcu_dft_exec_timed(tcu_dft_plan_t p, const void *in, void *out, int dir,
                        void *stream, void *const *events);
 

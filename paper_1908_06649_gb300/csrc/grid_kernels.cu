@@ -272,8 +272,9 @@ cudaError_t launch_extract_tiles(float *Ak, const float2 *tiles, long long side,
 }  // namespace tcu
 
 // ---------------------------------------------------------- mixed radix
-// The q-point pass of a mixed-radix transform n = q R^k (q = 2 .. 16, any
-// integer): the four-step split n = q x n2 with the q-point DFTs over the
+// The q-point pass of a mixed-radix transform n = q R^k as a launch of its own
+// (q = 5 .. 16, where q sub-transforms do not fit the next pass's items: mix_team
+// in tcu_dft.cu): the four-step split n = q x n2 with the q-point DFTs over the
 // stride-n2 columns done on the CUDA cores -- for q <= 16 a tensor-core
 // product would be mostly padding -- straight from the definition
 // y_k = sum_a x_a w_q^{a k}, then the inter-pass twiddle w_n^{k v} from the
@@ -319,9 +320,6 @@ cudaError_t launch_radix_q(int q, const float2 *x, float2 *out, long long batch,
                            int num_sms, cudaStream_t st) {
   const unsigned grid = grid_for(batch << log2n2, num_sms);
   switch (q) {
-    case 2: radix_q_kernel<2><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;
-    case 3: radix_q_kernel<3><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;
-    case 4: radix_q_kernel<4><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;
     case 5: radix_q_kernel<5><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;
     case 6: radix_q_kernel<6><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;
     case 7: radix_q_kernel<7><<<grid, kBlock, 0, st>>>(x, out, batch, log2n2, twA, twB, roots); break;

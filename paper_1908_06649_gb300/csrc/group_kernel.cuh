@@ -61,7 +61,17 @@ enum RowMode { kQF = 0, kUF = 1, kRQF = 2 };
 // output T[b n + v L + a], v < q, -> y[b n + v + k q]
 // kCols: one of several column passes of a 2-D transform, whose column
 // count, prefix and remaining rows are runtime values
-enum Role { kSingle = 0, kFirst = 1, kSecond = 2, kSecondQ = 4, kCols = 5 };
+// kFirstQ, kSecondQF: kFirst / kSecondQ of a mixed-radix transform with the
+// q-point pass done on the way in (mix_rows), q at run time
+enum Role {
+  kSingle = 0,
+  kFirst = 1,
+  kSecond = 2,
+  kSecondQ = 4,
+  kCols = 5,
+  kFirstQ = 6,
+  kSecondQF = 7
+};
 // What a column pass (the LP argument of a kCols kernel) does besides its
 // transforms: an inter-pass twiddle; a product with a spectrum; input rows
 // gathered as pairs of real columns from the windows of a real grid; output
@@ -90,7 +100,8 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // in SMEM, which leaves room for four; a radix-16 last pass of several runs
 // four too (measured faster than five: 0.165 instead of 0.181 ms for the
 // second pass of n = 16^4 x 1024), and so does a column pass (256 x 256 x
-// 1000 339 us against 363).  A radix-32 pass of two stages runs
+// 1000 339 us against 363); whole mixed-radix transforms run five (512 x
+// 130000 204 us against 216).  A radix-32 pass of two stages runs
 // four warpgroups whose slots hold A for half of K (the products of a stage
 // in two K halves); one-stage radix-32 passes (already near the copy rate),
 // the convolution row pass and the fused schedule keep whole-K slots, two
@@ -99,7 +110,7 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 __host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
   return R == 8    ? (S == 3 ? 5 : 8)
          : R == 32 ? (S >= 2 ? 4 : 2)
-                   : (ROLE != 0 && ROLE != 4 ? 4 : 5);
+                   : (ROLE != 0 && ROLE != 4 && ROLE != 7 ? 4 : 5);
 }
 __host__ __device__ constexpr int whole_k_nwg(int R, int ROLE, int S = 2) {
   return R == 32 ? 2 : (R == 16 ? 4 : pass_nwg(R, ROLE, S));
@@ -164,13 +175,19 @@ struct Geo {
   static constexpr long long OUT_STRIDE =
       ROLE == kSingle ? 1 : (1ll << (LOG2O + LOG2PRE));
   static constexpr long long OUT_VSTRIDE = ROLE == kSingle ? 0 : 1;
-  static constexpr bool STRIDED = ROLE == kFirst || RTC;
+  static constexpr bool STRIDED = ROLE == kFirst || ROLE == kFirstQ || RTC;
+  // the q-point pass of a mixed-radix transform on the way in: an item holds
+  // all q sequences of GG / q columns (FQ), or GG / q (rounded down) whole
+  // transforms (SQ)
+  static constexpr bool FQ = ROLE == kFirstQ, SQ = ROLE == kSecondQF;
+  static constexpr int QMAX = GG < 16 ? GG : 16;
+  static constexpr int MIX_ENTRIES = SQ ? (QMAX - 1) * L : 0;  // its twiddles, in SMEM
   // the sub-transforms' prefix count q is a runtime value (PRun::q)
-  static constexpr bool RTQ = ROLE == kSecondQ;
+  static constexpr bool RTQ = ROLE == kSecondQ || ROLE == kSecondQF;
   static constexpr int MODE_FIRST = STRIDED ? kUF : kQF;
   static constexpr int MODE_MID = kUF;
   static constexpr int MODE_LAST = ROLE == kSingle ? kRQF : kUF;
-  static constexpr bool TW_OUT = ROLE == kFirst;
+  static constexpr bool TW_OUT = ROLE == kFirst || ROLE == kFirstQ;
   // inter-pass twiddles staged by TMA per item (else read from the
   // L2-resident tables): measured faster for radix 16 and for the radix-8
   // team items; the one-warpgroup radix-8 items run faster with five
@@ -201,6 +218,11 @@ struct Geo {
 // Rows of a column pass's one-level twiddle table.
 constexpr int kLog2ColRows = 8;
 
+// The q-point pass of a mixed-radix transform.
+struct RootsQ {
+  float2 w[16];  // w_q^m, m < q, of the direction
+};
+
 // Runtime part of a pass.
 struct PRun {
   const float2 *in;
@@ -219,8 +241,14 @@ struct PRun {
   // process the items last to first: set on a pass that reads what the
   // previous pass wrote, whose latest output is still in L2
   int reverse;
-  // kSecondQ: the factor q of n = q R^S (sub-transforms per transform)
-  int q;
+  // kSecondQ: the factor q of n = q R^S (sub-transforms per transform).
+  // kFirstQ, kSecondQF: q, its log2 (kFirstQ: a power of two), the
+  // sub-transforms of an item (kSecondQF: a multiple of q), the roots, and the
+  // q-point pass's twiddles w_n^{k v}, v = vh 256 + vl, as mix_a [k][vl], mix_b
+  // [vh][k] (kFirstQ) or w_n^{k a} as mix_a [k - 1][a], 0 < k < q (kSecondQF)
+  int q, lq, subs;
+  const float2 *mix_a, *mix_b;
+  RootsQ roots;
   // kCols: log2 of the values after a row (rest n2), of the prefix P and of
   // the columns n2; its twiddles are tw_out[row of rest][k] (rows beyond
   // kColRows: tw_out[row mod kColRows][k] times tw_b[row / kColRows][k])
@@ -286,6 +314,16 @@ struct SmemLayout {
   static constexpr size_t BYTES = OFF_SCHED + 32 * NWG;
   static_assert(BYTES <= 227 * 1024, "shared memory budget");
 };
+
+// Items of a pass, and the first sub-transform of one.
+template <class G>
+__host__ __device__ __forceinline__ long long pass_items(const PRun &P) {
+  return G::SQ ? (P.U + P.subs - 1) / P.subs : (P.U + G::GG - 1) >> G::LOG2GG;
+}
+template <class G>
+__device__ __forceinline__ long long item_first(const PRun &P, long long item) {
+  return G::SQ ? item * P.subs : item << G::LOG2GG;
+}
 
 // log2 of the sub-transforms per sequence.
 template <class G>
@@ -513,9 +551,23 @@ __device__ __forceinline__ void load_d_row(const WG &w, float *d) {
 template <class G, bool HINT = false>
 __device__ __forceinline__ void issue_input(const PRun &P, const CUtensorMap *tm,
                                             long long item, const WG &w, uint64_t pol = 0) {
-  const long long u0 = item << G::LOG2GG;
+  const long long u0 = item_first<G>(P, item);
   const uint32_t dst = smem_u32(w.stg);
-  if (G::MODE_FIRST == kUF) {
+  if constexpr (G::FQ) {
+    // GG / q columns of each of the q sequences: staging [p][a][column]
+    const int lgc = G::LOG2GG - P.lq;
+    const long long c0 = item << lgc;
+    const long long b = (c0 >> G::LOG2UPER) << P.lq;
+    const int v0 = (int)(c0 & ((1ll << G::LOG2UPER) - 1));
+    if (elect_one()) {
+      mbar_expect_tx(w.bar_stg, G::GPTS * 8);
+      for (int p = 0; p < P.q; ++p)
+#pragma unroll
+        for (int a0 = 0; a0 < G::L; a0 += G::TMA_ROWS)
+          tma_load_3d(dst + (((p << G::LOG2L) + a0) << lgc) * 8, tm, 2 * v0, a0, (int)b + p,
+                      w.bar_stg);
+    }
+  } else if (G::MODE_FIRST == kUF) {
     // strided first pass: box of GG sub-transforms x L points
     const long long b = u0 >> log2_uper<G>(P);
     const int v0 = (int)(u0 & ((1ll << log2_uper<G>(P)) - 1));
@@ -532,7 +584,8 @@ __device__ __forceinline__ void issue_input(const PRun &P, const CUtensorMap *tm
   } else {
     // contiguous block of GG sub-transforms (the last item may be short)
     long long rem = P.U - u0;
-    if (rem > G::GG) rem = G::GG;
+    const int most = G::SQ ? P.subs : G::GG;
+    if (rem > most) rem = most;
     const uint32_t bytes = (uint32_t)(rem << G::LOG2L) * 8u;
     const long long b = u0 >> G::LOG2UPER;
     const long long v = u0 & ((1ll << G::LOG2UPER) - 1);
@@ -564,7 +617,8 @@ template <class G>
 __device__ __forceinline__ void issue_twiddles(const PRun &P, const CUtensorMap *tm,
                                                long long item, const WG &w) {
   if constexpr (G::TW_SMEM) {
-    const long long u0 = item << G::LOG2GG;
+    const int lgc = G::LOG2GG - (G::FQ ? P.lq : 0);  // log2 of the item's columns
+    const long long u0 = item << lgc;
     const long long v0 = u0 & ((1ll << G::LOG2UPER) - 1);
     const int vl0 = (int)(v0 & ((1 << G::LOG2VL) - 1));
     const uint32_t dst = smem_u32(w.tws);
@@ -572,10 +626,10 @@ __device__ __forceinline__ void issue_twiddles(const PRun &P, const CUtensorMap 
     const bool ok =
         !G::TW2L || in_range(w, boff + G::L - 1, (1ll << (G::LOG2UPER - G::LOG2VL)) << G::LOG2L);
     if (elect_one()) {
-      mbar_expect_tx(w.bar_tws, G::GPTS * 8 + (G::TW2L && ok ? G::L * 8 : 0));
+      mbar_expect_tx(w.bar_tws, (G::L * 8 << lgc) + (G::TW2L && ok ? G::L * 8 : 0));
 #pragma unroll
       for (int k0 = 0; k0 < G::L; k0 += G::TMA_ROWS)
-        tma_load_3d(dst + k0 * G::GG * 8, tm, 2 * vl0, k0, 0, w.bar_tws);
+        tma_load_3d(dst + (k0 * 8 << lgc), tm, 2 * vl0, k0, 0, w.bar_tws);
       if (G::TW2L && ok) tma_load_1d(smem_u32(w.twb), P.tw_b + boff, G::L * 8, w.bar_tws);
     }
     __syncwarp();
@@ -594,15 +648,220 @@ __device__ __forceinline__ void issue_stage(uint32_t slot, uint32_t img_addr,
   __syncwarp();
 }
 
+// ---- mixed radix: the q-point pass of n = q R^k on the way in.  In a pass of
+// its own it was an HBM round trip for q-point sums (2 16^4 x 500: 158 of
+// 487 us); here a thread takes the q staged values of one column at a time,
+// forms the q sums, multiplies by the twiddle and leaves them in the transpose
+// buffer (free until the first transposition), from
+// which the stage-1 rows are read.
+
+// kFirstQ: place of value a of sub-transform ul = (p, column) in the transpose
+// buffer: rows of GG values, p rotated by the row, so that the rows of a
+// half-warp's columns fall on different banks.
+template <class G>
+__device__ __forceinline__ int fq_index(const PRun &P, int a, int ul) {
+  return a * G::GG + (ul ^ ((a & (P.q - 1)) << (G::LOG2GG - P.lq)));
+}
+
+// z + x w, w = w_Q^m: a sum, a difference or a swap for the quarter turns.
+template <int Q0, int Q>
+__device__ __forceinline__ float2 add_root(const RootsQ &r, float2 z, float2 x, int m) {
+  if (m == 0) return make_float2(z.x + x.x, z.y + x.y);
+  if (2 * m == Q) return make_float2(z.x - x.x, z.y - x.y);
+  const float2 w = r.w[m * (Q0 / Q)];
+  if (4 * m == Q || 4 * m == 3 * Q)
+    return make_float2(fmaf(-x.y, w.y, z.x), fmaf(x.x, w.y, z.y));
+  return make_float2(fmaf(x.x, w.x, fmaf(-x.y, w.y, z.x)),
+                     fmaf(x.x, w.y, fmaf(x.y, w.x, z.y)));
+}
+
+// y[k SY] = sum over i < Q of x[i SX] w_Q^{i k}, from the definition (DEF, or a
+// prime Q), else as Q1 x Q2 (Cooley-Tukey): 15 = 3 x 5 takes half the operations.
+template <int Q0, int Q, int SX, int SY, bool DEF>
+__device__ __forceinline__ void dft_q(const RootsQ &r, const float2 *x, float2 *y) {
+  constexpr int Q1 = DEF                    ? Q
+                     : Q % 4 == 0 && Q > 4 ? 4
+                     : Q % 2 == 0           ? 2
+                     : Q % 3 == 0           ? 3
+                                            : Q;
+  constexpr int Q2 = Q / Q1;
+  if constexpr (Q2 == 1) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      float2 z = x[0];
+#pragma unroll
+      for (int i = 1; i < Q; ++i) z = add_root<Q0, Q>(r, z, x[i * SX], (i * k) % Q);
+      y[k * SY] = z;
+    }
+  } else {
+    // i = i1 Q2 + i2, k = k1 + Q1 k2
+    float2 t[Q];  // [k1][i2]
+#pragma unroll
+    for (int i2 = 0; i2 < Q2; ++i2) {
+      dft_q<Q0, Q1, Q2 * SX, Q2, DEF>(r, x + i2 * SX, t + i2);
+#pragma unroll
+      for (int k1 = 1; k1 < Q1; ++k1)
+        if (i2 > 0)
+          t[k1 * Q2 + i2] =
+              add_root<Q0, Q>(r, make_float2(0.f, 0.f), t[k1 * Q2 + i2], i2 * k1);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < Q1; ++k1) dft_q<Q0, Q2, 1, Q1 * SY, DEF>(r, t + k1 * Q2, y + k1 * SY);
+  }
+}
+
+// A strided pass's columns are taken UN at a time, all their values and twiddles
+// loaded before the first store (which a later load could not pass).  TF32 (PREC 1)
+// takes the sums from the definition: its products round their operands, and
+// the sums' own last bits would move them.
+template <class G, int PREC, int Q>
+__device__ __forceinline__ void mix_q(const PRun &P, const float2 *tw, long long item,
+                                      const WG &w) {
+  constexpr int UN = Q <= 4 ? 2 : 1;
+  constexpr bool DEF = PREC == 1;
+  const float2 one = make_float2(1.f, 0.f);
+  if constexpr (G::FQ && (Q & (Q - 1)) == 0 && 2 * Q <= (1 << G::LOG2R)) {
+    constexpr int LGC = G::LOG2GG - (Q == 2 ? 1 : Q == 4 ? 2 : Q == 8 ? 3 : 4);
+    constexpr int COLS = 1 << LGC;
+    constexpr int LVL = G::LOG2N > 8 ? 8 : G::LOG2N;
+    static_assert(G::L * COLS % (UN * G::ROWS) == 0, "whole groups of columns");
+    const long long v0 = (item << LGC) & ((1ll << G::LOG2UPER) - 1);
+#pragma unroll 1
+    for (int p0 = w.rho; p0 < G::L * COLS; p0 += UN * G::ROWS) {
+      float2 x[UN][Q], t[UN][Q];
+#pragma unroll
+      for (int n = 0; n < UN; ++n) {
+        const int pos = p0 + n * G::ROWS, a = pos >> LGC, c = pos & (COLS - 1);
+        const long long v = ((long long)a << G::LOG2UPER) + v0 + c;
+        const long long vl = v & ((1 << LVL) - 1), vh = v >> LVL;
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+          x[n][i] =
+              in_range(w, i * G::L * COLS + pos, G::GPTS) ? w.stg[i * G::L * COLS + pos] : one;
+#pragma unroll
+        for (int k = 1; k < Q; ++k) {
+          const long long ia = ((long long)k << LVL) + vl, ib = vh * Q + k;
+          t[n][k] = in_range(w, ia, (long long)Q << LVL) ? __ldg(P.mix_a + ia) : one;
+          if (G::LOG2N > 8 && in_range(w, ib, (long long)Q << (G::LOG2N - LVL)))
+            t[n][k] = cmul(t[n][k], __ldg(P.mix_b + ib));
+        }
+      }
+#pragma unroll
+      for (int n = 0; n < UN; ++n) {
+        const int pos = p0 + n * G::ROWS, a = pos >> LGC, c = pos & (COLS - 1);
+        float2 y[Q];
+        dft_q<Q, Q, 1, 1, DEF>(P.roots, x[n], y);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+          const int o = fq_index<G>(P, a, (k << LGC) | c);
+          if (in_range(w, o, G::GPTS)) w.buf[o] = k > 0 ? cmul(y[k], t[n][k]) : y[k];
+        }
+      }
+    }
+  }
+  // (radix 8 takes more than eight values only where they factor: mix_team)
+  constexpr bool FITS = G::LOG2R > 3 || Q <= 8 || (!DEF && Q != 11 && Q != 13);
+  if constexpr (G::SQ && Q <= G::QMAX && FITS) {
+    // whole transforms: staging and transpose buffer [transform][p][a]; in
+    // place where the two are one buffer
+    const int count = (P.subs / Q) << G::LOG2L;
+    for (int pos = w.rho; pos < count; pos += G::ROWS) {
+      const int a = pos & (G::L - 1), base = (pos >> G::LOG2L) * (Q * G::L) + a;
+      float2 x[Q], y[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        x[i] = in_range(w, base + i * G::L, G::GPTS) ? w.stg[base + i * G::L] : one;
+      dft_q<Q, Q, 1, 1, DEF>(P.roots, x, y);
+#pragma unroll
+      for (int k = 0; k < Q; ++k) {
+        if (k > 0)
+          y[k] = cmul(y[k], in_range(w, (k - 1) * G::L + a, G::MIX_ENTRIES)
+                                ? tw[(k - 1) * G::L + a]
+                                : one);
+        if (in_range(w, base + k * G::L, G::GPTS)) w.buf[base + k * G::L] = y[k];
+      }
+    }
+  }
+}
+
+// kFirstQ with q = 2: this thread's stage-1 row straight from the staging, both
+// values of a column read by both its threads; no barrier and no round trip
+// through the transpose buffer (2 16^4 x 500: the pass 274 -> 241 us; a launch of
+// its own and the strided pass 331).
+template <class G>
+__device__ __forceinline__ void staged_row_fq2(const PRun &P, long long item, const WG &w,
+                                               float2 *x) {
+  constexpr int R = 1 << G::LOG2R;
+  constexpr int JS = 1 << (G::LOG2L - G::LOG2R);
+  constexpr int LGC = G::LOG2GG - 1, COLS = 1 << LGC;
+  constexpr int LVL = G::LOG2N > 8 ? 8 : G::LOG2N;
+  int ul, q;
+  row_of<G>(kUF, w.rho, ul, q);
+  const int c = ul & (COLS - 1), k = ul >> LGC;
+  const int v = (int)((item << LGC) & ((1ll << G::LOG2UPER) - 1)) + c;
+  const float sign = k ? -1.f : 1.f;
+  const float2 one = make_float2(1.f, 0.f);
+  const float2 *ta = P.mix_a + (k << LVL), *tb = P.mix_b + k;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int a = j * JS + q, i = a * COLS + c, at = (a << G::LOG2UPER) + v;
+    const float2 x0 = in_range(w, i, G::GPTS) ? w.stg[i] : one;
+    const float2 x1 = in_range(w, G::L * COLS + i, G::GPTS) ? w.stg[G::L * COLS + i] : one;
+    float2 t = in_range(w, (k << LVL) + (at & ((1 << LVL) - 1)), 2 << LVL)
+                   ? __ldg(ta + (at & ((1 << LVL) - 1)))
+                   : one;
+    if (G::LOG2N > 8 && in_range(w, 2 * (at >> LVL) + k, 2ll << (G::LOG2N - LVL)))
+      t = cmul(t, __ldg(tb + 2 * (at >> LVL)));
+    x[j] = cmul(make_float2(fmaf(sign, x1.x, x0.x), fmaf(sign, x1.y, x0.y)), t);
+  }
+}
+
+template <class G, int PREC>
+__device__ __forceinline__ void mix_rows(const PRun &P, const float2 *tw, long long item,
+                                         const WG &w) {
+  switch (P.q) {
+    case 2:
+      if (!G::FQ) mix_q<G, PREC, 2>(P, tw, item, w);
+      break;
+    case 3: mix_q<G, PREC, 3>(P, tw, item, w); break;
+    case 4: mix_q<G, PREC, 4>(P, tw, item, w); break;
+    case 5: mix_q<G, PREC, 5>(P, tw, item, w); break;
+    case 6: mix_q<G, PREC, 6>(P, tw, item, w); break;
+    case 7: mix_q<G, PREC, 7>(P, tw, item, w); break;
+    case 8: mix_q<G, PREC, 8>(P, tw, item, w); break;
+    case 9: mix_q<G, PREC, 9>(P, tw, item, w); break;
+    case 10: mix_q<G, PREC, 10>(P, tw, item, w); break;
+    case 11: mix_q<G, PREC, 11>(P, tw, item, w); break;
+    case 12: mix_q<G, PREC, 12>(P, tw, item, w); break;
+    case 13: mix_q<G, PREC, 13>(P, tw, item, w); break;
+    case 14: mix_q<G, PREC, 14>(P, tw, item, w); break;
+    case 15: mix_q<G, PREC, 15>(P, tw, item, w); break;
+    case 16: mix_q<G, PREC, 16>(P, tw, item, w); break;
+    default: break;
+  }
+}
+
 // This thread's stage-1 row, from the staged input block.
 template <class G>
-__device__ __forceinline__ void staged_row(const WG &w, float2 *x) {
+__device__ __forceinline__ void staged_row(const PRun &P, const WG &w, float2 *x) {
   constexpr int R = 1 << G::LOG2R;
   int ul, q;
   row_of<G>(G::MODE_FIRST, w.rho, ul, q);
   constexpr int JS = 1 << (G::LOG2L - G::LOG2R);  // a = j * R^(S-1) + q
   const float2 zero = make_float2(0.f, 0.f);
-  if (G::MODE_FIRST == kUF) {
+  if constexpr (G::FQ) {
+    // the transpose buffer, as mix_rows left it: [a][ul ^ rotation of a]
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int i = fq_index<G>(P, j * JS + q, ul);
+      x[j] = in_range(w, i, G::GPTS) ? w.buf[i] : zero;
+    }
+  } else if constexpr (G::SQ) {
+    const int i0 = (ul << G::LOG2L) + q;  // transpose buffer [ul][a]
+    const float2 *p = w.buf + i0;
+#pragma unroll
+    for (int j = 0; j < R; ++j) x[j] = in_range(w, i0 + j * JS, G::GPTS) ? p[j * JS] : zero;
+  } else if (G::MODE_FIRST == kUF) {
     const int i0 = q * G::GG + ul;  // staging [a][ul]
     const float2 *p = w.stg + i0;
 #pragma unroll
@@ -789,7 +1048,7 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   constexpr int S = G::LOG2L / G::LOG2R;
   int ul, q;
   row_of<G>(G::MODE_LAST, w.rho, ul, q);
-  const long long u = (item << G::LOG2GG) + ul;
+  long long u = item_first<G>(P, item) + ul;
   float d[2 * R];
   load_d_row<G, PREC>(w, d);
   if constexpr (G::TW_SMEM) {
@@ -799,7 +1058,7 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
       w.fail = true;
     w.ph_tws ^= 1;
   }
-  if (u >= P.U) return;
+  if (u >= P.U || (G::SQ && ul >= P.subs)) return;
   int klow = 0, vq = q;
 #pragma unroll
   for (int i = 0; i < S - 1; ++i) {
@@ -826,6 +1085,17 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
     dst = P.out + b * (q << G::LOG2L) + v + klow * q;
     JS = q << (G::LOG2L - G::LOG2R);
   }
+  // an item's columns in the twiddle tile, and this one
+  const int lgc = G::LOG2GG - (G::FQ ? P.lq : 0), uc = G::FQ ? ul & ((1 << lgc) - 1) : ul;
+  if constexpr (G::FQ) {
+    // sequence p of the transform, column of the item
+    const long long c = (item << lgc) + uc, p = ul >> lgc;
+    b = c >> G::LOG2UPER;
+    v = c & ((1ll << G::LOG2UPER) - 1);
+    dst = P.out + (b << (G::LOG2N + P.lq)) + (p << G::LOG2UPER) + v +
+          ((long long)klow << (G::LOG2UPER + P.lq));
+    JS = 1ll << (G::LOG2UPER + P.lq + G::LOG2L - G::LOG2R);
+  }
   if constexpr (G::RTC) {
     // sequence b = (array, p): row (k P + p) of the array
     const int ls = P.lo + P.lp;
@@ -844,8 +1114,8 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   const bool ctwo = G::RTC_TW && P.tw_b != nullptr;
   // twiddle of output k = klow + j r^(S-1): table A staged as [k][ul] in SMEM,
   // or read from global [k][vl]; two-level: times B[vh][k]
-  const float2 *tws = w.tws + klow * G::GG + ul;
-  constexpr int TJS = G::GG << (G::LOG2L - G::LOG2R);
+  const float2 *tws = w.tws + (klow << lgc) + uc;
+  const int TJS = 1 << (lgc + G::LOG2L - G::LOG2R);
   const long long vl = v & ((1ll << G::LOG2VL) - 1), vh = v >> G::LOG2VL;
   const float2 *twg = P.tw_out + ((long long)klow << G::LOG2VL) + vl;
   constexpr long long TWG = 1ll << (G::LOG2VL + G::LOG2L - G::LOG2R);
@@ -858,7 +1128,7 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   const long long doff = dst - P.out;
   const long long out_elems =
       P.out_bmask == -1 ? (P.U << G::LOG2L) : ((P.out_bmask + 1) << G::LOG2NT);
-  const long long toff = klow * G::GG + ul, goff = ((long long)klow << G::LOG2VL) + vl;
+  const long long toff = (klow << lgc) + uc, goff = ((long long)klow << G::LOG2VL) + vl;
   const long long gboff = (vh << G::LOG2L) + klow;
   const float2 one = make_float2(1.f, 0.f);
   // The factors of a chunk of outputs (spectrum, twiddles) are loaded before
@@ -913,8 +1183,8 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
 // before the first epilogue barrier).  On entry the item's input copy has been issued.
 template <class G, int PREC, bool OUT_L2, class Mid>
 __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *tm_tw,
-                                             const float2 *tws, long long item, WG &w,
-                                             Mid &mid) {
+                                             const float2 *tws, const float2 *mix_tw,
+                                             long long item, WG &w, Mid &mid) {
   constexpr int R = 1 << G::LOG2R;
   constexpr int S = G::LOG2L / G::LOG2R;
   if constexpr (G::GATHER) {
@@ -924,9 +1194,26 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
     w.ph_stg ^= 1;
   }
   mid.after_load(w);
+  // whether the q-point sums pass through the transpose buffer
+  const bool mixed = G::SQ || (G::FQ && P.q > 2);
+  if (mixed) {
+    mix_rows<G, PREC>(P, mix_tw, item, w);
+    if (named_bar_or(w.bar_id, w.bar_count, w.fail)) {
+      w.fail = true;
+      return;
+    }
+    // the staging has been read
+    if (w.copy_lead) mid.issue(w);
+  }
   {
     float2 x[R];
-    staged_row<G>(w, x);
+    bool direct = false;
+    if constexpr (G::FQ) direct = !mixed;
+    if (direct) {
+      if constexpr (G::FQ) staged_row_fq2<G>(P, item, w, x);
+    } else {
+      staged_row<G>(P, w, x);
+    }
 #pragma unroll
     for (int c = 0; c < R; c += 8)
       split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
@@ -950,7 +1237,7 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
       issue_twiddles<G>(P, tm_tw, item, w);
       w.tws_inflight = true;
     }
-    if constexpr (!G::GATHER) mid.issue(w);
+    if (!G::GATHER && !mixed) mid.issue(w);
   }
   if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
   w.ph_mma ^= 1;
@@ -1020,7 +1307,7 @@ __device__ __forceinline__ void staged_row_half(const WG &w, float2 *x, int h) {
 #pragma unroll
   for (int j = 0; j < H; ++j) {
     const int i = i0 + (h * H + j) * JST;
-    x[j] = in_range(w, i, G::GPTS) ? w.stg[i] : zero;
+    x[j] = in_range(w, i, G::GPTS) ? w.stg[i] : zero;  // (a mixed pass: in place)
   }
 }
 
@@ -1059,7 +1346,8 @@ __device__ __forceinline__ void stage_rows_half(const PRun &P, const WG &w, int 
 
 template <class G, int PREC, class Mid>
 __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws,
-                                                long long item, WG &w, Mid &mid) {
+                                                const float2 *mix_tw, long long item, WG &w,
+                                                Mid &mid) {
   constexpr int R = 1 << G::LOG2R, H = R / 2;
   constexpr int S = G::LOG2L / G::LOG2R;
   static_assert(G::KS && S <= 2 && !G::TW_SMEM, "half-K items: radix 32, at most two stages");
@@ -1069,6 +1357,13 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
   } else {
     if (!mbar_wait_bounded(w.bar_stg, w.ph_stg)) w.fail = true;
     w.ph_stg ^= 1;
+  }
+  if constexpr (G::SQ) {
+    mix_rows<G, PREC>(P, mix_tw, item, w);
+    if (named_bar_or(w.bar_id, w.bar_count, w.fail)) {
+      w.fail = true;
+      return;
+    }
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -1318,7 +1613,7 @@ __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *t
     if constexpr (CONV == kRealConv)
       staged_half_row<G>(w, x);
     else
-      staged_row<G>(w, x);
+      staged_row<G>(P, w, x);
 #pragma unroll
     for (int c = 0; c < R; c += 8)
       split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
@@ -1499,18 +1794,20 @@ __global__ void __launch_bounds__(
       Geo<R, S, LO, ROLE, LP,
           TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>;
   static_assert(!CONV || ROLE == kSingle, "convolution rows are whole transforms");
-  using SM = SmemLayout<R, G::NWG, G::TW_ENTRIES, CONV ? G::TW_ENTRIES : 0, G::TW_SMEM, G::TWB,
-                        TW, G::KS>;
+  using SM = SmemLayout<R, G::NWG, G::TW_ENTRIES, CONV ? G::TW_ENTRIES : G::MIX_ENTRIES,
+                        G::TW_SMEM, G::TWB, TW, G::KS>;
   extern __shared__ __align__(1024) unsigned char smem[];
   float2 *tw = reinterpret_cast<float2 *>(smem + SM::OFF_TW1);
   float2 *tw_inv = reinterpret_cast<float2 *>(smem + SM::OFF_TW2);
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + SM::OFF_BAR);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mbar + 3 * G::NWG);
   const PRun &P = a.p[0];
-  // a convolution row pass also holds the inverse stage twiddles (p[1])
+  // a convolution row pass also holds the inverse stage twiddles (p[1]), a
+  // whole mixed-radix transform the q-point pass's
   kernel_setup_start<G::NWG, G::THREADS>(
       a.bimg, (int)(SM::IMG / 4), reinterpret_cast<float *>(smem), P.tw_stage, tw,
-      G::TW_ENTRIES, a.p[1].tw_stage, tw_inv, CONV ? G::TW_ENTRIES : 0, mbar, tmem_slot);
+      G::TW_ENTRIES, G::SQ ? P.mix_a : a.p[1].tw_stage, tw_inv,
+      CONV ? G::TW_ENTRIES : (G::SQ ? (P.q - 1) << G::LOG2L : 0), mbar, tmem_slot);
   WG w;
   init_wg<R, SM, G::GCOLS, TW>(w, 0, smem);  // TMEM slot set below
   // In a strided pass of two or more stages warp 1 issues the copies after
@@ -1518,14 +1815,14 @@ __global__ void __launch_bounds__(
   // 0's products, which the other warps otherwise wait for at the next
   // barrier (measured: these passes 1 % faster; the others, and one-stage
   // strided passes, slower)
-  if (ROLE == kFirst && S >= 2 && !G::KS && !CONV)
+  if ((ROLE == kFirst || ROLE == kFirstQ) && S >= 2 && !G::KS && !CONV)
     w.copy_lead = (threadIdx.x >> 5) % (4 * TW) == 1;
 #ifdef TCU_DFT_CHECKED
   w.err = a.err;
 #endif
 
   const int team = (threadIdx.x >> 7) / TW;
-  const long long nitems = (P.U + G::GG - 1) >> G::LOG2GG;
+  const long long nitems = pass_items<G>(P);
   const long long istride = (long long)gridDim.x * G::NTEAM;
   // team-major: with fewer items than SMs each CTA holds one item
   long long item = (long long)team * gridDim.x + blockIdx.x;
@@ -1547,12 +1844,12 @@ __global__ void __launch_bounds__(
     if constexpr (CONV != kNoConv)
       process_item_conv<G, PREC, CONV>(P, tw, tw_inv, phys(item), w, nx);
     else if constexpr (G::KS)
-      process_item_ks<G, PREC>(P, tw, phys(item), w, nx);
+      process_item_ks<G, PREC>(P, tw, tw_inv, phys(item), w, nx);
     else
       // a strided pass writes the next pass's input: L2-cached stores keep
       // its latest part for the next pass (which starts there), streaming
       // stores otherwise
-      process_item<G, PREC, ROLE == kFirst || ROLE == kCols>(P, &a.tm_tw, tw, phys(item), w, nx);
+      process_item<G, PREC, G::STRIDED>(P, &a.tm_tw, tw, tw_inv, phys(item), w, nx);
     item += istride;
   }
   if (w.fail && w.rho == 0) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);
@@ -1819,9 +2116,9 @@ __global__ void __launch_bounds__(
       }
     }
     if (pass == 0)
-      process_item<G1, PREC, true>(a.p[0], &a.tm_tw, tw1, item, w, nx);
+      process_item<G1, PREC, true>(a.p[0], &a.tm_tw, tw1, nullptr, item, w, nx);
     else
-      process_item<G2, PREC, false>(a.p[1], &a.tm_tw, tw2, item, w, nx);
+      process_item<G2, PREC, false>(a.p[1], &a.tm_tw, tw2, nullptr, item, w, nx);
     stg_pending = nx.n1_issued;
     if (w.fail) break;
     // the mailbox now names the next item; its completion is published
@@ -2103,7 +2400,7 @@ __device__ __forceinline__ void process_pair_item(const PRun &P, const float2 *t
   if (TYPE == 1) mid.after_load(w);
   {
     float2 x[R];
-    staged_row<G>(w, x);
+    staged_row<G>(P, w, x);
 #pragma unroll
     for (int c = 0; c < R; c += 8)
       split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,

@@ -23,7 +23,7 @@ constexpr int kHostChunks = 16;  // pipeline depth of the host-buffer path
 
 struct PassPlan {
   int s;            // stages
-  int role;         // kSingle, kFirst (strided) or kSecond (last of several)
+  int role;         // Role
   int so;           // kFirst: stages after this pass; kSecond: stages before
   int sp;           // kFirst: stages before this pass
   int lo;           // log2: columns of a strided pass / points before the last
@@ -43,7 +43,8 @@ struct PassPlan {
   int q;
   RootsQ roots[2];
   bool mixed;
-  int qrt;          // kSecondQ: the factor q of n = q r^s (runtime prefix count)
+  int qrt;          // kSecondQ, kSecondQF, kFirstQ: the factor q (at run time)
+  int subs;         // kSecondQF: sub-transforms of an item, a multiple of q
   int tw;           // warpgroups per item (teams for the 3-stage radix-8 passes)
 };
 
@@ -155,6 +156,8 @@ struct tcu_dft_plan_s {
   tcu::host::PassPlan pass[tcu::host::kMaxPasses];
   float *bimg[2];          // [dir index] hi | lo | scaled hi | scaled lo images
   float2 *scratch[2];      // intermediates (or the fused ring in scratch[0])
+  // mixed radix: pass 1 takes the q-point pass 0 on its way in (one launch)
+  bool mix;
   // fused two-pass schedule
   bool fused;
   // one HBM pass on cluster pairs (scratch[0]: two slots per cluster)
@@ -190,7 +193,7 @@ int plan_stages(int r, int k, int st[kMaxPasses]);
 // r = 32).  Any other q = 2 .. 16 (odd factors): one pass with a runtime
 // q, k = 1..3 for r = 8, k = 1..2 for r = 16 and 32.  Returns the number of
 // passes (0: not such an n) and fills the passes.
-int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]);
+int plan_mixed(int r, long long n, long long batch, int precision, PassPlan pass[kMaxPasses]);
 // Warpgroups per item of pass pp (its role and stages are set).
 int team_size(int r, const PassPlan &pp);
 // Role, neighbouring stage counts, size and row maps of pass `pi`.

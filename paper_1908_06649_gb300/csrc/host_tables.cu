@@ -296,11 +296,12 @@ void pass_twiddles(long long L, long long n2, int sign, std::vector<float2> &A,
   }
 }
 
-// TMA map of table A of a strided pass (boxes of GG columns x L rows).
+// TMA map of table A of a strided pass (boxes of an item's columns x L rows: GG,
+// or GG / q of each of q sequences).
 bool twiddle_map(CUtensorMap *m, const float2 *A, int r, const PassPlan &pp) {
   const long long L = 1ll << pp.log2L, n2 = 1ll << pp.lo;
   const long long VL = n2 > 256 ? 256 : n2;
-  const long long gg = (128ll * pp.tw * r) >> pp.log2L;
+  const long long gg = ((128ll * pp.tw * r) >> pp.log2L) >> (pp.role == kFirstQ ? pp.lp : 0);
   return encode_map(m, A, VL, L, 1, L * VL, (int)gg, L < 256 ? (int)L : 256);
 }
 
@@ -309,7 +310,7 @@ bool twiddle_map(CUtensorMap *m, const float2 *A, int r, const PassPlan &pp) {
 bool input_map(CUtensorMap *m, const void *in, const tcu_dft_plan_s *p, const PassPlan &pp,
                long long batch) {
   const long long L = 1ll << pp.log2L, n2 = 1ll << pp.lo, pre = 1ll << pp.lp;
-  const long long gg = (128ll * pp.tw * p->r) >> pp.log2L;
+  const long long gg = ((128ll * pp.tw * p->r) >> pp.log2L) >> (pp.role == kFirstQ ? pp.lp : 0);
   return encode_map(m, in, n2, L, batch * pre, L * n2, (int)gg, L < 256 ? (int)L : 256);
 }
 

@@ -74,9 +74,6 @@ cudaError_t launch_spectrum_product(float2 *x, const float2 *spec, long long bat
                                     long long n, int num_sms, cudaStream_t st);
 
 // The q-point first pass of a mixed-radix transform (grid_kernels.cu).
-struct RootsQ {
-  float2 w[16];  // w_q^m, m < q, of the direction
-};
 cudaError_t launch_radix_q(int q, const float2 *x, float2 *out, long long batch, int log2n2,
                            const float2 *twA, const float2 *twB, const RootsQ &roots,
                            int num_sms, cudaStream_t st);
@@ -88,12 +85,12 @@ cudaError_t launch_pass_bf16_r32(int prec, int s, int lo, int role, int lp,
 cudaError_t launch_pass_bf16_r16(int prec, int s, int lo, int role, int lp,
                                  const GArgs &a, int num_sms, cudaStream_t st);
 // Mixed-radix warpgroup passes (kernels_mixed_r*.cu): same arguments as
-// launch_pass_r*.
-cudaError_t launch_pass_mixed_r8(int prec, int s, int lo, int role, int lp, const GArgs &a,
+// launch_pass_r*, and the warpgroups of an item.
+cudaError_t launch_pass_mixed_r8(int prec, int s, int lo, int role, int lp, int tw, const GArgs &a,
                                  int num_sms, cudaStream_t st);
-cudaError_t launch_pass_mixed_r16(int prec, int s, int lo, int role, int lp, const GArgs &a,
+cudaError_t launch_pass_mixed_r16(int prec, int s, int lo, int role, int lp, int tw, const GArgs &a,
                                   int num_sms, cudaStream_t st);
-cudaError_t launch_pass_mixed_r32(int prec, int s, int lo, int role, int lp, const GArgs &a,
+cudaError_t launch_pass_mixed_r32(int prec, int s, int lo, int role, int lp, int tw, const GArgs &a,
                                   int num_sms, cudaStream_t st);
 
 }  // namespace tcu

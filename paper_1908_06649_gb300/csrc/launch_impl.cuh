@@ -11,14 +11,14 @@ template <int R, int PREC, int S, int LO, int ROLE, int LP>
 cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, LO, ROLE, LP>;
   const size_t sm =
-      SmemLayout<R, G::NWG, G::TW_ENTRIES, 0, G::TW_SMEM, G::TWB, 1, G::KS>::BYTES;
+      SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, 1, G::KS>::BYTES;
   cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   // one CTA per SM, each item on its own SM while there are fewer items
   // than SMs (latency), several per SM otherwise
-  const long long nitems = (a.p[0].U + G::GG - 1) >> G::LOG2GG;
+  const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
   dft_pass_kernel<R, PREC, S, LO, ROLE, LP><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
   return cudaGetLastError();
@@ -29,12 +29,12 @@ cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
 template <int R, int PREC, int S, int LO, int ROLE, int LP, int TW>
 cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, LO, ROLE, LP, team_nwg(R), TW>;
-  const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, 0, G::TW_SMEM, G::TWB, TW>::BYTES;
+  const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, TW>::BYTES;
   cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
-  const long long nitems = (a.p[0].U + G::GG - 1) >> G::LOG2GG;
+  const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
   dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>
       <<<(unsigned)grid, G::THREADS, sm, st>>>(a);
@@ -57,7 +57,7 @@ cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
-  const long long nitems = (a.p[0].U + G::GG - 1) >> G::LOG2GG;
+  const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
   dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
   return cudaGetLastError();

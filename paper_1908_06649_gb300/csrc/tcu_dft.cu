@@ -85,15 +85,52 @@ int plan_stages(int r, int k, int st[kMaxPasses]) {
   return P;
 }
 
+// Warpgroups of an item of the pass that takes the q-point sums of n = q r^k on
+// its way in; 0: the q-point pass stays a launch of its own.  A whole transform
+// (k stages in one pass) needs q sub-transforms of an item's GG = 128 TW r / r^k;
+// two warpgroups an item where they use 15 or more than 8 of 16 (n = 1280 x
+// 50000: 237 us against 267 at 5 of 8; n = 768 x 130000, 15 of 16 against 6 of 8:
+// 382 us against 330, so one for q = 3).  At radix 8 eight warpgroups share the
+// registers, and sums of more than eight values gain only where they factor
+// (15 8^2 x 50000: 283 -> 217 us, 13 8^2 x 60000: 274 -> 302) and not from the
+// definition (TF32, 15 8^2: 279 -> 308) nor at 9 of 16.  The strided pass of
+// several holds GG / q columns of each of the q sequences, at least four (32-byte
+// runs).
+int mix_team(int r, int k, int q, int precision) {
+  if (r == 16) return k == 2 ? (q == 5 || q > 8 ? 2 : 1) : (k == 4 ? (q <= 4 ? 2 : 0) : 1);
+  if (r == 32) return k == 2 && q > 4 ? 0 : 1;
+  if (k == 3) return q <= 8 ? 4 : 0;
+  if (q <= 8) return 1;
+  return precision == TCU_DFT_3XTF32 && q != 11 && q != 13 && (k == 1 || q != 9) ? 1 : 0;
+}
+
+// Pass 1 of a mixed-radix plan with the q-point pass 0 on its way in.
+void take_mix(int r, int k, int precision, PassPlan pass[kMaxPasses]) {
+  PassPlan &pp = pass[1];
+  const int q = pass[0].q, tw = mix_team(r, k, q, precision);
+  if (!tw) return;
+  pp.role = pp.last ? kSecondQF : kFirstQ;
+  pp.qrt = q;
+  pp.tw = tw;
+  if (pp.last) {
+    const int gg = (128 * tw * r) >> pp.log2L;
+    pp.lo = 0;
+    pp.subs = gg / q * q;
+  }
+  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, tw);
+}
+
 // Mixed radix n = q r^k (q < r a power of two; the base case of the
 // recursion is a DFT of size q < sqrt(m)): a CUDA-core q-point first pass,
 // then the r^k-point transforms of its q rows in one or two tensor-core
-// passes (stage split as plan_stages).  Instantiated: k = 2..4 for r = 8
+// passes (stage split as plan_stages), the first of which takes the q-point
+// sums on its way in where they fit its items (take_mix).  Instantiated: k = 2..4 for r = 8
 // and 16, k = 2..3 for r = 32.  Returns the number of passes (0: not such
 // an n) and fills the passes.
 // n = q r^k with q = 2 .. 16 not a power of two: the q-point pass, then one
 // tensor-core pass over the q rows (role kSecondQ, q at run time).
-int plan_mixed_q(int r, long long n, long long batch, PassPlan pass[kMaxPasses]) {
+int plan_mixed_q(int r, long long n, long long batch, int precision,
+                 PassPlan pass[kMaxPasses]) {
   const int log2r = ilog2(r);
   const int kmax = r == 8 ? 3 : 2;
   int k = 0;
@@ -132,13 +169,15 @@ int plan_mixed_q(int r, long long n, long long batch, PassPlan pass[kMaxPasses])
   pp.modes[2] = kUF;
   pp.tw = team_size(r, pp);
   pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
+  take_mix(r, k, precision, pass);
   return 2;
 }
 
-int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]) {
+int plan_mixed(int r, long long n, long long batch, int precision,
+               PassPlan pass[kMaxPasses]) {
   const int log2r = ilog2(r);
   if (n < 1) return 0;
-  if (n & (n - 1)) return plan_mixed_q(r, n, batch, pass);
+  if (n & (n - 1)) return plan_mixed_q(r, n, batch, precision, pass);
   const int log2n = ilog2(n), k = log2n / log2r, lq = log2n - k * log2r;
   const int kmax = r == 32 ? 3 : 4;
   if (lq == 0 || k < 2 || k > kmax) return 0;
@@ -181,6 +220,7 @@ int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]) {
     pp.tw = team_size(r, pp);
     pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   }
+  take_mix(r, k, precision, pass);
   return 1 + tc;
 }
 
@@ -188,13 +228,11 @@ int plan_mixed(int r, long long n, long long batch, PassPlan pass[kMaxPasses]) {
 // strided side (an item of 512 rows holds 8 sub-transforms of 512 points, so
 // that side moves 64-byte runs; items of one warpgroup move 16-byte runs, half
 // a sector: 8^7 x 32 last pass 567 -> 229 us, 8^8 x 4 passes 2 and 3
-// 562 + 629 -> 271 + 225 us, 512^2 x 200 463 -> 378 us).  After a prefix of
-// two a run is 16 bytes either way: one warpgroup (2 8^3 x 65536: 274 us
-// against 322).  2 for 16^3 in one pass, else 1.
+// 562 + 629 -> 271 + 225 us, 512^2 x 200 463 -> 378 us).  2 for 16^3 in one
+// pass, else 1.
 int team_size(int r, const PassPlan &pp) {
   if (r == 16 && pp.role == kSingle && pp.s == 3) return 2;
-  if (r != 8 || pp.s != 3 || pp.role == kSingle) return 1;
-  return pp.role == kSecond && pp.lo == 1 ? 1 : 4;
+  return r == 8 && pp.s == 3 && pp.role != kSingle ? 4 : 1;
 }
 
 // Role, neighbouring stage counts, size and row maps of pass `pi`.
@@ -258,9 +296,10 @@ void free_plan(tcu_dft_plan_s *p) {
 cudaError_t pass_dispatch(int r, int prec, const PassPlan &pp, const GArgs &a, int num_sms,
                           cudaStream_t st) {
   if (pp.mixed) {
-    if (r == 8) return launch_pass_mixed_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
-    if (r == 16) return launch_pass_mixed_r16(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
-    return launch_pass_mixed_r32(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
+    const int lp = pp.role == kFirstQ ? 0 : pp.lp;  // its prefix is a runtime value
+    if (r == 8) return launch_pass_mixed_r8(prec, pp.s, pp.lo, pp.role, lp, pp.tw, a, num_sms, st);
+    if (r == 16) return launch_pass_mixed_r16(prec, pp.s, pp.lo, pp.role, lp, pp.tw, a, num_sms, st);
+    return launch_pass_mixed_r32(prec, pp.s, pp.lo, pp.role, lp, pp.tw, a, num_sms, st);
   }
   if (prec_bf16(prec)) {
     if (r == 8) return launch_pass_bf16_r8(prec, pp.s, pp.lo, pp.role, pp.lp, a, num_sms, st);
@@ -305,8 +344,16 @@ PRun group_pass(const tcu_dft_plan_s *p, int pi, int di, const float2 *in, float
   // every second pass runs its items last to first: it starts on what the
   // pass before wrote last, still in L2 (measured 0.5-2.5 % per pass; not on
   // team passes, where it measured 1.5 % slower)
-  g.reverse = (pi & 1) && pp.tw == 1;
+  g.reverse = ((pi - p->mix) & 1) && pp.tw == 1;
   g.q = pp.qrt;
+  if (p->mix && pi == 1) {
+    const PassPlan &pq = p->pass[0];
+    g.lq = ilog2(pp.qrt);
+    g.subs = pp.subs;
+    g.mix_a = pq.tw_a[di];
+    g.mix_b = pq.tw_b[di];
+    g.roots = pq.roots[di];
+  }
   // the inverse's last stage uses the F images scaled by 1/n
   g.last_img = (pp.last && inverse) ? 2 * (prec_bf16(p->precision) ? 8 : 16) * p->r * p->r : 0;
   return g;
@@ -319,8 +366,24 @@ void dir_tables(const tcu_dft_plan_s *p, int d, DirTables &t) {
     const PassPlan &pp = p->pass[pi];
     t.stage[pi] = stage_twiddles(p->r, pp.q ? 1 : pp.s, sign);
     // the q-point pass has L = q rows (any q); a tensor-core pass L = r^s
-    if (pp.role == kFirst)
+    if (pp.q && p->mix && p->pass[1].role == kSecondQF) {
+      // w_n^{k a} as [k - 1][a], a < r^s: the products of the two-level tables
+      // of the q-point pass
+      const long long len = 1ll << pp.lo, VL = len > 256 ? 256 : len;
+      std::vector<float2> A, B;
+      pass_twiddles(pp.q, len, sign, A, B);
+      for (long long k = 1; k < pp.q; ++k)
+        for (long long a = 0; a < len; ++a) {
+          float2 w = A[(size_t)(k * VL + a % VL)];
+          if (len > VL) {
+            const float2 z = B[(size_t)(a / VL * pp.q + k)];
+            w = make_float2(fmaf(w.x, z.x, -(w.y * z.y)), fmaf(w.x, z.y, w.y * z.x));
+          }
+          t.A[pi].push_back(w);
+        }
+    } else if (pp.role == kFirst || pp.role == kFirstQ) {
       pass_twiddles(pp.q ? pp.q : (1ll << pp.log2L), 1ll << pp.lo, sign, t.A[pi], t.B[pi]);
+    }
   }
 }
 
@@ -410,10 +473,13 @@ int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
   for (int pi = 0; pi < p->npasses; ++pi) {
     const NvtxRange range(kRange[pi]);
     const PassPlan &pp = p->pass[pi];
-    const float2 *src = (pi == 0) ? (const float2 *)in : p->scratch[pi - 1] + off;
-    float2 *dst = pp.last ? (float2 *)out : p->scratch[pi] + off;
+    // launch l of the plan (a mixed-radix plan's first two passes may be one)
+    const int l = pi - p->mix;
+    const float2 *src = (l <= 0) ? (const float2 *)in : p->scratch[l - 1] + off;
+    float2 *dst = pp.last ? (float2 *)out : p->scratch[l < 0 ? 0 : l] + off;
     if (events && cudaEventRecord((cudaEvent_t)events[pi], st) != cudaSuccess)
       return TCU_DFT_ERR_CUDA;
+    if (pp.q && p->mix) continue;
     if (pp.q) {
       if (launch_radix_q(pp.q, src, dst, count, pp.lo, pp.tw_a[di], pp.tw_b[di],
                          pp.roots[di], p->num_sms, st) != cudaSuccess)
@@ -423,7 +489,7 @@ int exec_impl(tcu_dft_plan_t p, const void *in, void *out, int dir,
     GArgs g;
     memset(&g, 0, sizeof(g));
     g.p[0] = group_pass(p, pi, di, src, dst, -1, -1, inverse, count);
-    if (pp.role == kFirst) {
+    if (pp.role == kFirst || pp.role == kFirstQ) {
       if (!input_map(&g.tm_in, src, p, pp, count)) return TCU_DFT_ERR_CUDA;
       g.tm_tw = pp.tw_map[di];
     }
@@ -491,7 +557,7 @@ tcu_dft_plan_t tcu_dft_plan_ex(int64_t n, int64_t batch, int32_t sqrt_m,
   PassPlan mixed[kMaxPasses];
   memset(mixed, 0, sizeof(mixed));
   const bool is_mixed = m != n;
-  const int npasses = is_mixed ? plan_mixed(r, n, batch, mixed)
+  const int npasses = is_mixed ? plan_mixed(r, n, batch, precision, mixed)
                                : (k >= 1 ? plan_stages(r, k, st) : 0);
   // the BF16 modes are instantiated for n = r^k (no mixed radix)
   if (npasses == 0 || (long long)batch * n > (1ll << 40) ||
@@ -520,9 +586,11 @@ tcu_dft_plan_t tcu_dft_plan_ex(int64_t n, int64_t batch, int32_t sqrt_m,
   p->npasses = npasses;
   p->device = dev;
   p->num_sms = prop.multiProcessorCount;
-  if (is_mixed)
+  if (is_mixed) {
     for (int pi = 0; pi < npasses; ++pi) p->pass[pi] = mixed[pi];
-  else
+    p->mix = mixed[1].role == kFirstQ || mixed[1].role == kSecondQF;
+  }
+  if (!is_mixed)
     for (int pi = 0; pi < npasses; ++pi) pass_geometry(p->pass[pi], pi, npasses, st, k, r, n, batch);
   int rc = TCU_DFT_OK;
   for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
@@ -532,7 +600,7 @@ tcu_dft_plan_t tcu_dft_plan_ex(int64_t n, int64_t batch, int32_t sqrt_m,
     for (int pi = 0; pi < npasses && rc == TCU_DFT_OK; ++pi) {
       PassPlan &pp = p->pass[pi];
       rc = upload(&pp.tw_stage[d], t.stage[pi]);
-      if (rc == TCU_DFT_OK && pp.role == kFirst) {
+      if (rc == TCU_DFT_OK && (pp.role == kFirst || pp.role == kFirstQ)) {
         rc = upload(&pp.tw_a[d], t.A[pi]);
         if (rc == TCU_DFT_OK && !t.B[pi].empty()) rc = upload(&pp.tw_b[d], t.B[pi]);
         if (rc == TCU_DFT_OK && !pp.q && !twiddle_map(&pp.tw_map[d], pp.tw_a[d], r, pp))
@@ -588,7 +656,7 @@ tcu_dft_plan_t tcu_dft_plan_ex(int64_t n, int64_t batch, int32_t sqrt_m,
         rc = TCU_DFT_ERR_OOM;
       }
     }
-    for (int i = 0; i < npasses - 1 && rc == TCU_DFT_OK; ++i)
+    for (int i = 0; i < npasses - 1 - p->mix && rc == TCU_DFT_OK; ++i)
       if (dev_malloc((void **)&p->scratch[i], (size_t)scratch_tf * n * sizeof(float2)) !=
           cudaSuccess) {
         cudaGetLastError();
@@ -731,7 +799,7 @@ int tcu_dft_plan_passes(int64_t n, int32_t sqrt_m, int32_t *stages) {
   } else {
     PassPlan mixed[kMaxPasses];
     memset(mixed, 0, sizeof(mixed));
-    np = plan_mixed(r, n, 1, mixed);
+    np = plan_mixed(r, n, 1, TCU_DFT_3XTF32, mixed);
     for (int i = 0; i < np; ++i) st[i] = mixed[i].s;
   }
   for (int i = 0; i < np; ++i) stages[i] = st[i];

@@ -121,3 +121,19 @@ def test_real_tiles(pkg, r, side, k):
     plan.check()
     assert torch.equal(Ad, got)
     plan.destroy()
+
+
+# mixed radix with the q-point sums on the way into a tensor-core pass: whole
+# transforms (every q that fits, items that use all, some or one transform's
+# sub-transforms of theirs, last items of one), and the strided pass of several
+@pytest.mark.parametrize("r,q,k,batch", [
+    (16, 2, 2, 5), (16, 3, 2, 1), (16, 3, 2, 4), (16, 4, 2, 3), (16, 5, 2, 4), (16, 6, 2, 1),
+    (16, 7, 2, 2), (16, 8, 2, 3), (16, 9, 2, 1), (16, 11, 2, 2), (16, 14, 2, 1), (16, 15, 2, 3),
+    (16, 3, 1, 43), (16, 15, 1, 9), (16, 2, 3, 3), (16, 8, 3, 1), (16, 2, 4, 1), (16, 4, 4, 1),
+    (16, 8, 4, 1), (8, 3, 1, 43), (8, 13, 1, 10), (8, 15, 1, 9), (8, 2, 2, 9), (8, 9, 2, 3),
+    (8, 12, 2, 2), (8, 15, 2, 1), (8, 2, 3, 5), (8, 3, 3, 3), (8, 7, 3, 1), (8, 10, 3, 1),
+    (8, 2, 4, 3), (8, 4, 4, 1), (32, 3, 1, 43), (32, 14, 1, 10), (32, 2, 2, 3), (32, 3, 2, 2),
+    (32, 4, 2, 1), (32, 5, 2, 1), (32, 16, 2, 1), (32, 2, 3, 1), (32, 8, 3, 1), (32, 16, 3, 1)])
+@pytest.mark.parametrize("prec,inverse", [(3, False), (3, True), (1, False)])
+def test_mixed_on_the_way_in(pkg, r, q, k, batch, prec, inverse):
+    _check_1d(pkg, q * r ** k, batch, r, prec, inverse, seed=q + k)
