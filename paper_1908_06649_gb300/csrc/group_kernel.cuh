@@ -1802,6 +1802,12 @@ __global__ void __launch_bounds__(
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + SM::OFF_BAR);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mbar + 3 * G::NWG);
   const PRun &P = a.p[0];
+  // Launched with programmatic serialization: the stream's next pass kernel may
+  // take this one's place on an SM as it leaves, and sets itself up (barriers,
+  // TMEM, the plan's constant tables) while others finish.  Nothing another
+  // kernel writes is read, and nothing is written, before wait_prior_grids,
+  // which every thread passes, so completion is transitive along a stream.
+  launch_dependents();
   // a convolution row pass also holds the inverse stage twiddles (p[1]), a
   // whole mixed-radix transform the q-point pass's
   kernel_setup_start<G::NWG, G::THREADS>(
@@ -1830,6 +1836,7 @@ __global__ void __launch_bounds__(
   // item: position in this CTA's sequence; phys: the item processed there
   // (team passes always run forward: no reversal code in them)
   auto phys = [&](long long i) { return TW == 1 && P.reverse ? nitems - 1 - i : i; };
+  wait_prior_grids();
   // the first input copy of team 0 leaves with the tables (warp 0 set up its
   // mbarriers), the other teams' after the CTA barrier
   // (gathered columns: every thread copies its own row, after the barrier)

@@ -7,21 +7,49 @@
 
 namespace tcu {
 
+// A pass kernel's launch: `sm` bytes of shared memory and, with `beside`, set up
+// beside the stream's previous kernel (programmatic serialization; the kernel
+// waits for it before it touches data), which takes 2-3 us off every launch:
+// n = 65536 x 64 30.6 -> 26.2 us a call, 4096^2 stencils 138 -> 131.
+inline cudaError_t launch_serial(void (*kernel)(const GArgs), long long grid, int threads,
+                                 size_t sm, bool beside, const GArgs &a, cudaStream_t st) {
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = beside ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+// Long radix-8 passes are launched after the kernel before them: CTAs that take
+// the SMs in the order they fall free left these passes 1-2 % slower (n = 32768 x
+// 4096: 780 us against 796, 4096 x 16384 342 against 346: 54 and more items a
+// team; 32768 x 1500, 39 items: 293 us against 289 beside).
+template <class G>
+bool launch_beside(long long nitems, long long grid) {
+  return G::LOG2R > 3 || nitems <= 45 * grid * G::NTEAM;
+}
+
 template <int R, int PREC, int S, int LO, int ROLE, int LP>
 cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, LO, ROLE, LP>;
   const size_t sm =
       SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, 1, G::KS>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
-  if (e != cudaSuccess) return e;
   // one CTA per SM, each item on its own SM while there are fewer items
   // than SMs (latency), several per SM otherwise
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
-  dft_pass_kernel<R, PREC, S, LO, ROLE, LP><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_serial(dft_pass_kernel<R, PREC, S, LO, ROLE, LP>, grid, G::THREADS, sm,
+                       launch_beside<G>(nitems, grid), a, st);
 }
 
 // A team pass: items of TW warpgroups (128 TW rows), team_nwg(R) warpgroups
@@ -30,15 +58,10 @@ template <int R, int PREC, int S, int LO, int ROLE, int LP, int TW>
 cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, LO, ROLE, LP, team_nwg(R), TW>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, TW>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
-  if (e != cudaSuccess) return e;
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
-  dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>
-      <<<(unsigned)grid, G::THREADS, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_serial(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>, grid,
+                       G::THREADS, sm, launch_beside<G>(nitems, grid), a, st);
 }
 
 #define TCU_TEAM_CASE_L(S, LO, ROLE, LP, TW)                                             \
@@ -53,14 +76,10 @@ template <int R, int PREC, int S, int CONV>
 cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
   using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, kSingle, S)>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::TW_ENTRIES, false, 0>::BYTES;
-  cudaError_t e = cudaFuncSetAttribute(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
-  if (e != cudaSuccess) return e;
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
-  dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV><<<(unsigned)grid, G::THREADS, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_serial(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV>, grid, G::THREADS, sm,
+                       launch_beside<G>(nitems, grid), a, st);
 }
 
 #define TCU_ROWCONV_CASE(S)                                                         \

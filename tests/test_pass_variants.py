@@ -137,3 +137,45 @@ def test_real_tiles(pkg, r, side, k):
 @pytest.mark.parametrize("prec,inverse", [(3, False), (3, True), (1, False)])
 def test_mixed_on_the_way_in(pkg, r, q, k, batch, prec, inverse):
     _check_1d(pkg, q * r ** k, batch, r, prec, inverse, seed=q + k)
+
+
+def test_launches_beside_one_another(pkg):
+    # pass kernels are set up while the kernel before them runs: a chain of
+    # calls that read and overwrite what the last ones wrote, of one to three
+    # launches each and with other kernels and table copies between, gives the
+    # same bits with and without a synchronisation after every call, on the
+    # default and on another stream
+    import torch
+    n, batch = 4096, 32
+    x0 = torch.from_numpy(inputs.make("normal", n, batch, seed=3)).cuda().reshape(-1)
+    a = pkg.Plan(4096, 32, 16, 3)          # one launch
+    b = pkg.Plan(65536, 2, 16, 3)          # two
+    c = pkg.Plan(8192, 16, 16, 3)          # q-point sums on the way in, two
+    d = pkg.Plan2(64, 64, 32, 8, 3)        # columns and rows
+    s = pkg.StencilPlan(512, 3, 16, 3)     # spectrum, three passes
+    w3 = [[0.0, 0.1, 0.0], [0.15, 0.5, 0.15], [0.0, 0.1, 0.0]]
+
+    def chain(sync):
+        x, y = x0.clone(), torch.empty_like(x0)
+        for i in range(6):
+            for f in (lambda: a.forward(x, y), lambda: b.inverse(y, y), lambda: c.forward(y, x),
+                      lambda: x.mul_(0.5), lambda: d.inverse(x, y),
+                      lambda: pkg.exec_noalloc(y, x, 256 if i & 1 else 512, 512 if i & 1 else 256,
+                                               16 if i & 1 else 8, 3),
+                      lambda: s.apply(torch.view_as_real(x).reshape(-1),
+                                      torch.view_as_real(y).reshape(-1), w3x3=w3),
+                      lambda: a.inverse(y, x)):
+                f()
+                if sync:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return x
+
+    ref = chain(True)
+    assert torch.isfinite(torch.view_as_real(ref)).all()
+    assert torch.equal(chain(False), ref)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        assert torch.equal(chain(False), ref)
+    for p in (a, b, c, d, s):
+        p.check()
+        p.destroy()
