@@ -451,7 +451,11 @@ __host__ __device__ constexpr int img_bytes(int R, int PREC) {
 // representable in TF32) and lo = v - hi is exact in fp32.  TF32: hi rounded
 // to nearest.  BF16 modes: hi = bf16 rounding of v, lo = bf16 rounding of
 // v - hi (exact in fp32 before rounding), packed two per column.
-template <int PREC>
+// PACK: lo of both parts by one packed subtraction, one instruction in four of
+// the split: taken in the three-stage passes, which issue and shared-memory
+// latency bound (16^3 x 16384 228 -> 222 us, last pass of 8^5 x 4096 449 -> 435,
+// 8^3 x 100000 151 -> 147); the strided two-stage passes were 1-2 % slower so.
+template <int PREC, bool PACK = false>
 __device__ __forceinline__ void split_store8(const float2 *x, uint32_t col_hi,
                                              uint32_t col_lo) {
   if constexpr (is_bf16(PREC)) {
@@ -479,8 +483,14 @@ __device__ __forceinline__ void split_store8(const float2 *x, uint32_t col_hi,
         const float hy = __uint_as_float(__float_as_uint(x[j].y) & 0xFFFFE000u);
         vh[2 * j] = hx;
         vh[2 * j + 1] = hy;
-        vl[2 * j] = x[j].x - hx;
-        vl[2 * j + 1] = x[j].y - hy;
+        if (PACK) {
+          const float2 l = sub2(x[j], make_float2(hx, hy));
+          vl[2 * j] = l.x;
+          vl[2 * j + 1] = l.y;
+        } else {
+          vl[2 * j] = x[j].x - hx;
+          vl[2 * j + 1] = x[j].y - hy;
+        }
       } else {
         vh[2 * j] = tf32_rna(x[j].x);
         vh[2 * j + 1] = tf32_rna(x[j].y);
@@ -958,7 +968,7 @@ __device__ __forceinline__ void stage_rows(const PRun &P, const WG &w) {
     }
 #pragma unroll
     for (int c8 = 0; c8 < CH; c8 += 8)
-      split_store8<PREC>(row + c8, w.slot + w.lane_off + a_cols8(PREC) * (c + c8) / 8,
+      split_store8<PREC, (S > 2)>(row + c8, w.slot + w.lane_off + a_cols8(PREC) * (c + c8) / 8,
                          w.slot + G::Q + w.lane_off + a_cols8(PREC) * (c + c8) / 8);
   }
 }
@@ -1216,7 +1226,7 @@ __device__ __forceinline__ void process_item(const PRun &P, const CUtensorMap *t
     }
 #pragma unroll
     for (int c = 0; c < R; c += 8)
-      split_store8<PREC>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
+      split_store8<PREC, (S > 2)>(x + c, w.slot + w.lane_off + a_cols8(PREC) * c / 8,
                          w.slot + G::Q + w.lane_off + a_cols8(PREC) * c / 8);
   }
   // the row is in TMEM: this thread's places of the staging are free again

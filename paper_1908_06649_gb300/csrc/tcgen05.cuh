@@ -269,6 +269,18 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
          | ((uint32_t)(M >> 4) << 24);
 }
 
+// a - b of both parts in one packed instruction (each rounded as by itself).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  union {
+    float2 f;
+    unsigned long long u;
+  } x, y, z;
+  x.f = a;
+  y.f = b;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(z.u) : "l"(x.u), "l"(y.u));
+  return z.f;
+}
+
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
