@@ -216,9 +216,11 @@ int col_stages(int r, int k, long long n2, int precision, int st[kMaxPasses]) {
   return P;
 }
 
-// The columns' tables: the F images scaled by 1/n, and per column pass
+// The columns' tables: the F images scaled by 1/n (unscaled ones also to
+// *conv_img, a convolution row pass's), and per column pass
 // its geometry, stage twiddles and inter-pass twiddles [row of rest][k].
-int make_cols(tcu_dft2_plan_s *p, const int *st, long long n) {
+int make_cols(tcu_dft2_plan_s *p, const int *st, long long n,
+              std::vector<float> *conv_img = nullptr) {
   const int log2r = ilog2(p->r);
   int rc = TCU_DFT_OK;
   long long pre = 1;
@@ -258,6 +260,8 @@ int make_cols(tcu_dft2_plan_s *p, const int *st, long long n) {
     std::vector<float> img;
     build_images(p->r, d == 0 ? -1 : 1, n, p->precision, img);
     rc = upload(&p->bimg[d], img);
+    // hi and lo of each direction (the first two images)
+    if (conv_img) conv_img->insert(conv_img->end(), img.begin(), img.begin() + img.size() / 2);
   }
   return rc;
 }
@@ -412,15 +416,9 @@ int make_two_pass(tcu_dft2_plan_s *p, int k1, int k2, long long row_len, long lo
   w.swz_tab = choose_swizzle(r, w.s, w.modes, w.tw);
   std::vector<float> conv_img;
   p->ncol = 1;
-  int rc = make_cols(p, &k1, p->n1 * row_len);
-  for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d) {
-    const int sign = d == 0 ? -1 : 1;
-    std::vector<float> img;
-    build_images(r, sign, p->n1 * row_len, p->precision, img);
-    // hi and lo of this direction (the first two images)
-    conv_img.insert(conv_img.end(), img.begin(), img.begin() + img.size() / 2);
-    rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, sign));
-  }
+  int rc = make_cols(p, &k1, p->n1 * row_len, &conv_img);
+  for (int d = 0; d < 2 && rc == TCU_DFT_OK; ++d)
+    rc = upload(&w.tw_stage[d], stage_twiddles(r, w.s, d == 0 ? -1 : 1));
   if (rc == TCU_DFT_OK) rc = upload(&p->cimg, conv_img);
   if (rc == TCU_DFT_OK &&
       (dev_malloc((void **)&p->scratch, (size_t)(p->batch * p->n1 * p->n2) * sizeof(float2)) !=

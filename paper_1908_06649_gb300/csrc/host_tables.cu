@@ -275,6 +275,7 @@ unsigned long long choose_swizzle(int r, int S, const int modes[3], int team) {
       bc = c;
       best = t;
     }
+    if (c <= 1.0) break;  // conflict free: no later candidate is better
   }
   return best;
 }

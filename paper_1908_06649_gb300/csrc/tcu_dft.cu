@@ -117,7 +117,6 @@ void take_mix(int r, int k, int precision, PassPlan pass[kMaxPasses]) {
     pp.lo = 0;
     pp.subs = gg / q * q;
   }
-  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, tw);
 }
 
 // Mixed radix n = q r^k (q < r a power of two; the base case of the
@@ -168,8 +167,8 @@ int plan_mixed_q(int r, long long n, long long batch, int precision,
   pp.modes[1] = kUF;
   pp.modes[2] = kUF;
   pp.tw = team_size(r, pp);
-  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   take_mix(r, k, precision, pass);
+  pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   return 2;
 }
 
@@ -218,9 +217,9 @@ int plan_mixed(int r, long long n, long long batch, int precision,
     pp.modes[1] = kUF;
     pp.modes[2] = kUF;
     pp.tw = team_size(r, pp);
+    if (i == 0) take_mix(r, k, precision, pass);
     pp.swz_tab = choose_swizzle(r, pp.s, pp.modes, pp.tw);
   }
-  take_mix(r, k, precision, pass);
   return 1 + tc;
 }
 
