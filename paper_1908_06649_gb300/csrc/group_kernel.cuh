@@ -344,8 +344,8 @@ struct WG {
   int rho;            // this thread's row within the item (0 .. 128 TW - 1)
   bool wg_lead;       // warp 0 of its warpgroup: issues the warpgroup's products
   bool team_lead;     // warp 0 of the team: runs the schedule
-  bool copy_lead;     // issues the team's copies: warp 0 of the team, or warp 1
-                      // in the strided passes of two or more stages
+  bool copy_lead;     // issues the team's copies after the first: warp 0 of the team,
+                      // or warp 1 in the passes that dft_pass_kernel names
   float2 *buf;        // SMEM transpose buffer
   float2 *stg;        // SMEM input staging (one item)
   float2 *tws;        // SMEM twiddle staging (one item)
@@ -1397,7 +1397,7 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
                                        w.bar_mma);
     }
     // one stage: the staging has been read and no transpose follows
-    if (S == 1 && h == 1 && w.team_lead) mid.issue(w);
+    if (S == 1 && h == 1 && w.copy_lead) mid.issue(w);
     if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
     w.ph_mma ^= 1;
     fence_after_sync();
@@ -1421,7 +1421,7 @@ __device__ __forceinline__ void process_item_ks(const PRun &P, const float2 *tws
         issue_stage_half<R, PREC, G::QA>(h, w.slot, w.img_addr + P.last_img, w.bar_mma);
       }
       // the transpose buffer (shared with the staging) has been read
-      if (h == 1 && (G::GATHER || w.team_lead)) mid.issue(w);
+      if (h == 1 && (G::GATHER || w.copy_lead)) mid.issue(w);
       if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
       w.ph_mma ^= 1;
       fence_after_sync();
@@ -1639,7 +1639,7 @@ __device__ __forceinline__ void process_item_conv(const PRun &P, const float2 *t
     fence_after_sync();
     issue_stage<R, PREC>(w.slot, w.img_addr, w.bar_mma);
   }
-  if (w.team_lead) mid.issue(w);
+  if (w.copy_lead) mid.issue(w);
   if (!mbar_wait_bounded(w.bar_mma, w.ph_mma)) w.fail = true;
   w.ph_mma ^= 1;
   fence_after_sync();
@@ -1826,12 +1826,16 @@ __global__ void __launch_bounds__(
       CONV ? G::TW_ENTRIES : (G::SQ ? (P.q - 1) << G::LOG2L : 0), mbar, tmem_slot);
   WG w;
   init_wg<R, SM, G::GCOLS, TW>(w, 0, smem);  // TMEM slot set below
-  // In a strided pass of two or more stages warp 1 issues the copies after
-  // the first one (the inter-pass twiddles and the next input), beside warp
-  // 0's products, which the other warps otherwise wait for at the next
-  // barrier (measured: these passes 1 % faster; the others, and one-stage
-  // strided passes, slower)
-  if ((ROLE == kFirst || ROLE == kFirstQ) && S >= 2 && !G::KS && !CONV)
+  // Warp 1 issues the copies after the first one (the inter-pass twiddles and
+  // the next input), beside warp 0's products, which the other warps otherwise
+  // wait for at the next barrier, where that measured faster: strided passes of
+  // two or more stages (1 %), half-K items (n = 1024 x 65536 173 -> 168 us), one
+  // pass of three stages (16^3 x 16384 222 -> 215, 8^3 x 100000 147 -> 144),
+  // convolution rows (radix-8 stencil of 4096^2 348 -> 335) and whole
+  // mixed-radix transforms on one warpgroup (192 x 200000 146 -> 142); not the
+  // last passes (three-stage radix-8 teams 435 -> 496) nor one-stage strided ones
+  if (((ROLE == kFirst || ROLE == kFirstQ) && S >= 2) || G::KS || CONV ||
+      (ROLE == kSingle && S == 3) || (G::SQ && TW == 1))
     w.copy_lead = (threadIdx.x >> 5) % (4 * TW) == 1;
 #ifdef TCU_DFT_CHECKED
   w.err = a.err;
