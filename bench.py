@@ -457,9 +457,12 @@ def run_grid(args):
         tiles, Nt, B = pkg.stencil_tiles(side, k, r)
         points = tiles * Nt * Nt
         passes = 3
-        # weights: place, 2-D DFT (2), power, inverse (2); kernel W': place,
-        # 2-D DFT (2); tiles: gather, convolution (3), extract
-        launches = 14
+        # 3xTF32 with tiles of one pass per axis: real tiles, columns gathered,
+        # rows, columns scattered; up to 24 steps the spectrum in one launch.
+        # Otherwise weights: place, 2-D DFT (2), power, inverse (2); kernel W':
+        # place, 2-D DFT (2); and complex tiles: gather, convolution (3), extract
+        real = args.precision == 3 and Nt <= {8: 512, 16: 256, 32: 1024}[r]
+        launches = (4 if k <= 24 else 12) if real else 14
         unit = "Gupdates/s"
         metric = ("linear stencil grid-point updates/s (side^2 x steps), "
                   "%d^2 grid x %d steps, 1xGB300" % (side, k))
@@ -496,15 +499,18 @@ def run_grid(args):
     ms = t0.elapsed_time(t1) / K
     cpu = None if args.no_cpu_baseline else grid_cpu_baseline(args, g)
     if args.grid == "stencil":
-        # whole step: the three convolution passes (16 B per tile point each),
-        # the gather (tile points written, the grid read once) and the
-        # extract (one tile point read and one grid point written per cell);
-        # the weight and kernel-spectrum transforms are tiny
+        # whole step.  Real tiles (4 B per tile point): gathered columns
+        # written, rows read and written, columns read; the grid read and
+        # written once.  Complex tiles: the three convolution passes (16 B per
+        # tile point each), the gather (tile points written, the grid read
+        # once) and the extract (one tile point read and one grid point
+        # written per cell).  The weight and kernel-spectrum steps are tiny
         S = float(side * side)
-        step_bytes = 48.0 * points + 8.0 * points + 4.0 * S + 8.0 * S + 4.0 * S
+        step_bytes = (16.0 * points + 8.0 * S if real else
+                      48.0 * points + 8.0 * points + 4.0 * S + 8.0 * S + 4.0 * S)
         achieved = step_bytes / (ms * 1e-3) / 1e9
-        kname = ("whole step (%d launches: weights, kernel spectrum, gather, 3 "
-                 "convolution passes, extract), %.2f GB algorithmic" % (launches, step_bytes / 1e9))
+        kname = ("whole step (%d launches: kernel spectrum, gather, convolution "
+                 "rows, scatter), %.2f GB algorithmic" % (launches, step_bytes / 1e9))
     else:
         achieved = 16.0 * points / (ms / passes * 1e-3) / 1e9
         kname = "average pass launch (%d pass launches per step)" % passes

@@ -229,9 +229,10 @@ int tcu_dft_exec_noalloc(int64_t n, int64_t batch, int32_t sqrt_m, int32_t preci
  * every row and of every column; Lemma 1 reduces stencils to batched
  * convolutions computed through it).  Arrays are row-major n1 x n2
  * complex64, batch-major (x[(b n1 + i) n2 + j]), 16-byte aligned, caller
- * owned.  n1 and n2 are powers of sqrt_m of at most one warpgroup pass each
- * (sqrt_m^2 for 16 and 32, 8^3 for 8) with n1 * n2 >= 128 sqrt_m.  Forward
- * unscaled; inverse with the conjugate exponent and 1/(n1 n2).
+ * owned.  n1 and n2 are powers of sqrt_m with a 1-D plan each.  In the TF32
+ * modes axes of at most one warpgroup pass (sqrt_m^2 for 16 and 32, 8^3 for 8)
+ * with n1 * n2 >= 128 sqrt_m take two passes, columns then rows; the others
+ * the rows' 1-D plan and up to three strided column passes.  Forward unscaled; inverse with the conjugate exponent and 1/(n1 n2).
  * tcu_dft2_plan allocates its tables and one batch-size scratch array and
  * returns NULL with tcu_dft_last_error() set on error (ERR_INVALID,
  * ERR_UNSUPPORTED, ERR_CUDA, ERR_OOM).  The exec calls are asynchronous on
