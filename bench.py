@@ -458,11 +458,11 @@ def run_grid(args):
         points = tiles * Nt * Nt
         passes = 3
         # 3xTF32 with tiles of one pass per axis: real tiles, columns gathered,
-        # rows, columns scattered; up to 24 steps the spectrum in one launch.
+        # rows, columns scattered; up to 20 steps the spectrum in one launch.
         # Otherwise weights: place, 2-D DFT (2), power, inverse (2); kernel W':
         # place, 2-D DFT (2); and complex tiles: gather, convolution (3), extract
         real = args.precision == 3 and Nt <= {8: 512, 16: 256, 32: 1024}[r]
-        launches = (4 if k <= 24 else 12) if real else 14
+        launches = (4 if k <= 20 else 12) if real else 14
         unit = "Gupdates/s"
         metric = ("linear stencil grid-point updates/s (side^2 x steps), "
                   "%d^2 grid x %d steps, 1xGB300" % (side, k))

@@ -51,33 +51,58 @@ __global__ void cpow_kernel(float2 *g, long long count, int k) {
 // periodic grid, directly: w[-a mod N][-b mod N] = W[k + a][k + b] are the
 // coefficients of P^k (Lemma 2), so its DFT at (f1, f2) is P(x, y)^k with
 // x = w_N^{-f1}, y = w_N^{-f2} (N >= 2 k + 1: nothing wraps).  In fp64, rounded
-// once: the k-th power multiplies a relative error of P by k.  A few dozen
-// fp64 operations a point and one launch, where placing P, its transform, the
-// power, the inverse, placing W' and its transform were nine (40 us).
+// once: the k-th power multiplies a relative error of P by k.  Bound by the few
+// fp64 units (and the launch): a thread takes ROWS rows of one column, whose
+// sums over b it forms once, and their powers side by side.  Two up to 256^2,
+// four above (calls on 1000^2, radix 16: 35.6 us with a point a thread, 31.0
+// with two, 32.4 with four; radix 32, tiles of 1024^2: 97.8 with one in this
+// form, 87.5, 81.7).  Placing P, its transform, the power, the inverse, placing
+// W' and its transform were nine launches, 40 us.
+template <int ROWS>
 __global__ void stencil_spectrum_kernel(float2 *S, const double2 *roots, int N, Stencil3 w,
                                         int k) {
-  const int count = (N / 2 + 1) * N;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    const double2 x = roots[e / N], y = roots[e % N];  // w_N^{-f}
-    double2 r[3];  // sum over b of w[a][b] y^b
+  const int rows = N / 2 + 1, groups = (rows + ROWS - 1) / ROWS;
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < groups * N;
+       g += gridDim.x * blockDim.x) {
+    const int f2 = g % N, f1 = g / N * ROWS;
+    const double2 y = roots[f2];  // w_N^{-f}
+    double2 r[3];                 // sum over b of w[a][b] y^b
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
       const double lo = w.w[3 * a], hi = w.w[3 * a + 2];
       r[a] = make_double2(fma(lo + hi, y.x, (double)w.w[3 * a + 1]), (hi - lo) * y.y);
     }
-    // x^-1 r[0] + r[1] + x r[2]
-    double2 base;
-    base.x = fma(x.x, r[0].x + r[2].x, fma(x.y, r[0].y - r[2].y, r[1].x));
-    base.y = fma(x.x, r[0].y + r[2].y, fma(x.y, r[2].x - r[0].x, r[1].y));
-    double2 acc = make_double2(1.0, 0.0);
+    // x^-1 r[0] + r[1] + x r[2] = Re x (r[2] + r[0]) + i Im x (r[2] - r[0]) + r[1]
+    const double2 sum = make_double2(r[0].x + r[2].x, r[0].y + r[2].y);
+    const double2 dif = make_double2(r[2].x - r[0].x, r[0].y - r[2].y);
+    double2 base[ROWS], acc[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const double2 x = roots[min(f1 + i, N / 2)];
+      base[i].x = fma(x.x, sum.x, fma(x.y, dif.y, r[1].x));
+      base[i].y = fma(x.x, sum.y, fma(x.y, dif.x, r[1].y));
+    }
+    bool first = true;
     for (int m = k;;) {
-      if (m & 1)
-        acc = make_double2(fma(acc.x, base.x, -acc.y * base.y),
-                           fma(acc.x, base.y, acc.y * base.x));
+      if (m & 1) {
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i)
+          acc[i] = first ? base[i]
+                         : make_double2(fma(acc[i].x, base[i].x, -acc[i].y * base[i].y),
+                                        fma(acc[i].x, base[i].y, acc[i].y * base[i].x));
+        first = false;
+      }
       m >>= 1;
       if (!m) break;
-      base = make_double2(fma(base.x, base.x, -base.y * base.y), 2.0 * base.x * base.y);
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i)
+        base[i] = make_double2(fma(base[i].x, base[i].x, -base[i].y * base[i].y),
+                               2.0 * base[i].x * base[i].y);
     }
-    S[e] = make_float2((float)acc.x, (float)acc.y);
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+      if (f1 + i < rows)
+        S[(f1 + i) * N + f2] = make_float2((float)acc[i].x, (float)acc[i].y);
   }
 }
 
@@ -216,12 +241,16 @@ cudaError_t launch_cpow(float2 *g, long long count, int k, int num_sms, cudaStre
 
 cudaError_t launch_stencil_spectrum(float2 *S, const double2 *roots, long long N,
                                     const Stencil3 &w, int k, int num_sms, cudaStream_t st) {
-  // one point per thread in small blocks, over all SMs (their few fp64 units
-  // bound it)
-  const long long blocks = ((N / 2 + 1) * N + 63) / 64;
+  // small blocks, over all SMs
+  const int rows = N > 256 ? 4 : 2;
+  const long long groups = (N / 2 + rows) / rows;
+  const long long blocks = (groups * N + 63) / 64;
   const long long cap = 16ll * num_sms;
-  stencil_spectrum_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 64, 0, st>>>(S, roots,
-                                                                                 (int)N, w, k);
+  const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
+  if (rows == 4)
+    stencil_spectrum_kernel<4><<<grid, 64, 0, st>>>(S, roots, (int)N, w, k);
+  else
+    stencil_spectrum_kernel<2><<<grid, 64, 0, st>>>(S, roots, (int)N, w, k);
   return cudaGetLastError();
 }
 

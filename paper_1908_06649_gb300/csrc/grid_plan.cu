@@ -78,12 +78,12 @@ struct tcu_stencil_plan_s {
 };
 
 // Steps up to which a real-tile plan evaluates the kernel's spectrum directly:
-// one launch instead of nine (a grid of 1000^2, 16 steps: 114 -> 45 us), and
+// one launch instead of nine (a grid of 1000^2, 16 steps: 114 -> 31 us), and
 // more exact (error of the output 7.9e-6 -> 1.3e-6).  Beyond, the spectrum
 // comes from the transforms of Lemma 2, as tcu_stencil_weights' weights do:
 // their error grows with k (about 5e-7 k of the output), and results stay
 // within 2e-5 of theirs on either side of the line.
-constexpr int kClosedSteps = 24;
+constexpr int kClosedSteps = 20;
 
 namespace {
 
