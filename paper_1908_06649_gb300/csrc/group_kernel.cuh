@@ -1817,7 +1817,6 @@ __global__ void __launch_bounds__(
   // TMEM, the plan's constant tables) while others finish.  Nothing another
   // kernel writes is read, and nothing is written, before wait_prior_grids,
   // which every thread passes, so completion is transitive along a stream.
-  launch_dependents();
   // a convolution row pass also holds the inverse stage twiddles (p[1]), a
   // whole mixed-radix transform the q-point pass's
   kernel_setup_start<G::NWG, G::THREADS>(
@@ -1856,6 +1855,12 @@ __global__ void __launch_bounds__(
   // (gathered columns: every thread copies its own row, after the barrier)
   if (!G::GATHER && team == 0 && w.team_lead) nx.issue(w);
   const uint32_t tbase = kernel_setup_finish(tmem_slot);
+  // Only now, with this CTA's TMEM its own: a CTA of the next kernel that fits
+  // beside this one then waits in its allocation for this one to leave.  Let in
+  // earlier it could take the columns first and wait for this kernel, which would
+  // wait for them without a limit (today no two of these CTAs share an SM, by
+  // registers or by shared memory; nothing here rests on that).
+  launch_dependents();
   w.slot = tbase + (uint32_t)((threadIdx.x >> 7) * G::GCOLS);
   if (G::GATHER || (team != 0 && w.team_lead)) nx.issue(w);
   // the tables have landed (the same answer in every thread of the team)
