@@ -352,7 +352,7 @@ struct WG {
   float2 *twb;        // SMEM row of twiddle table B (two-level tables)
   uint32_t ph_mma, ph_stg, ph_tws;
   bool fail;
-  bool tws_inflight;  // warp 0: a twiddle copy has not been waited on
+  bool tws_inflight;  // copy_lead's warp: a twiddle copy has not been seen to land
 #ifdef TCU_DFT_CHECKED
   int *err;           // error word: index violations are recorded at once
 #endif
@@ -1725,15 +1725,30 @@ __device__ __forceinline__ bool wait_tables(uint64_t *mbar, int nwg) {
   return mbar_wait_bounded(smem_u32(mbar + 3 * nwg + 1), 0);
 }
 
-// Leave: wait (bounded) for any copy still landing in this warpgroup's
-// staging, then free TMEM.
-__device__ __forceinline__ void kernel_teardown(uint32_t tbase, const WG &w, bool stg_pending,
-                                                bool tws_pending) {
-  // the first lane of the warp that issued the copies
+// Wait (bounded) until nothing is landing under a mbarrier of copies: whichever
+// phase it is in completes when an outstanding copy has landed (with none
+// outstanding it stays, and the limit ends the wait).  A thread's own phase bit
+// would not do: it is a phase ahead when the wait for that very copy ran out.
+__device__ __forceinline__ void drain_barrier(uint32_t bar) {
+  mbar_wait_bounded(bar, mbar_try_wait(bar, 0) ? 1 : 0, kDrainNs);
+}
+
+// A kernel whose wait ran out leaves early: one thread a team (stg, tws: whether
+// copies of its staging, of its twiddles may be outstanding) and one for the tables
+// wait for what is still landing in this CTA's shared memory, whoever issued it.
+__device__ __forceinline__ void drain_copies(const WG &w, bool stg, bool tws, uint64_t *mbar,
+                                             int nwg) {
   if (w.copy_lead && (threadIdx.x & 31) == 0) {
-    if (stg_pending) mbar_wait_bounded(w.bar_stg, w.ph_stg);
-    if (tws_pending) mbar_wait_bounded(w.bar_tws, w.ph_tws);
+    if (stg) drain_barrier(w.bar_stg);
+    if (tws) drain_barrier(w.bar_tws);
   }
+  if (threadIdx.x == 0 && w.fail) mbar_wait_bounded(smem_u32(mbar + 3 * nwg + 1), 0, kDrainNs);
+}
+
+// Leave: copies still landing after a failure, then free TMEM.
+__device__ __forceinline__ void kernel_teardown(uint32_t tbase, const WG &w, bool stg, bool tws,
+                                                uint64_t *mbar, int nwg) {
+  drain_copies(w, stg, tws, mbar, nwg);
   fence_before_sync();
   __syncthreads();
   if ((threadIdx.x >> 5) == 0) {
@@ -1777,7 +1792,8 @@ struct StaticNext {
   const PRun &P;
   const CUtensorMap *tm;
   long long next, nitems;
-  bool issued;  // a copy for `next` is in flight
+  bool issued;  // copy_lead's warp: its last issue() started a copy (before its
+                // first: the first item's, which warp 0 starts)
   // one warp, converged -- or, for gathered columns, every thread
   __device__ void issue(const WG &w) {
     issued = next < nitems;
@@ -1845,7 +1861,7 @@ __global__ void __launch_bounds__(
   const long long istride = (long long)gridDim.x * G::NTEAM;
   // team-major: with fewer items than SMs each CTA holds one item
   long long item = (long long)team * gridDim.x + blockIdx.x;
-  StaticNext<G, CONV> nx{P, &a.tm_in, item, nitems, false};
+  StaticNext<G, CONV> nx{P, &a.tm_in, item, nitems, item < nitems};
   // item: position in this CTA's sequence; phys: the item processed there
   // (team passes always run forward: no reversal code in them)
   auto phys = [&](long long i) { return TW == 1 && P.reverse ? nitems - 1 - i : i; };
@@ -1879,9 +1895,10 @@ __global__ void __launch_bounds__(
     item += istride;
   }
   if (w.fail && w.rho == 0) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);
-  // on failure a copy issued for the next item may still be landing
+  // on failure a copy for the item or the next may still be landing
   if (G::GATHER) cp_async_wait_all();
-  kernel_teardown(tbase, w, !G::GATHER && w.fail && nx.issued, w.fail && w.tws_inflight);
+  kernel_teardown(tbase, w, !G::GATHER && w.fail && nx.issued, w.fail && w.tws_inflight, mbar,
+                  G::NWG);
 }
 
 // ------------------------------------------------------- fused two passes
@@ -2119,7 +2136,6 @@ __global__ void __launch_bounds__(
   if (!wait_tables(mbar, NWG)) f = true;
   if (named_bar_or(w.bar_id, w.bar_count, f)) w.fail = true;
 
-  bool stg_pending = false;
   while (!w.fail) {
     const long long item = box->item;
     const int pass = box->pass, chunk = box->chunk;
@@ -2145,7 +2161,6 @@ __global__ void __launch_bounds__(
       process_item<G1, PREC, true>(a.p[0], &a.tm_tw, tw1, nullptr, item, w, nx);
     else
       process_item<G2, PREC, false>(a.p[1], &a.tm_tw, tw2, nullptr, item, w, nx);
-    stg_pending = nx.n1_issued;
     if (w.fail) break;
     // the mailbox now names the next item; its completion is published
     // during the next item (after its first barrier), or below
@@ -2157,7 +2172,7 @@ __global__ void __launch_bounds__(
   named_bar_or(w.bar_id, w.bar_count, false);
   if (w.team_lead) nx.publish_pending();
   if (w.rho == 0 && w.fail) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);
-  kernel_teardown(tbase, w, w.fail && stg_pending, w.fail && w.tws_inflight);
+  kernel_teardown(tbase, w, w.fail, w.fail && w.tws_inflight, mbar, NWG);
 }
 
 // ------------------------------------------ one HBM pass on cluster pairs
@@ -2565,7 +2580,6 @@ __global__ void __launch_bounds__(
   if (!wait_tables(mbar, NWG)) w.fail = true;
   // a uniform failure state before the first barrier
   if (named_bar_or(w.bar_id, w.bar_count, w.fail)) w.fail = true;
-  bool stg_pending = nx.issued;
   while (nx.cur.valid && !w.fail) {
     nx.nxt = pair_decode(pos + NWG, H, J);
     if (nx.cur.type == 0) {
@@ -2583,7 +2597,6 @@ __global__ void __launch_bounds__(
       process_pair_item<G2, PREC, 1>(prun[1], tw2, nx.gitem(nx.cur), w, nx);
       if (named_bar_or(w.bar_id, w.bar_count, w.fail)) w.fail = true;
     }
-    stg_pending = nx.issued;
     if (w.fail) break;
     pos += NWG;
     nx.cur = nx.nxt;
@@ -2598,7 +2611,6 @@ __global__ void __launch_bounds__(
         w.fail = true;
         break;
       }
-      stg_pending = true;
     }
   }
   // a last publication (after the last item nobody waits for it, but the
@@ -2607,10 +2619,7 @@ __global__ void __launch_bounds__(
   if (w.fail && w.rho == 0) atomicCAS(a.err, 0, TCU_DFT_ERR_TIMEOUT);
   // leave: copies of this warpgroup still landing (on failure), then the
   // cluster -- the peer may arrive on this CTA's barriers until it is done
-  if (w.rho == 0 && w.fail) {
-    if (stg_pending) mbar_wait_bounded(w.bar_stg, w.ph_stg);
-    if (w.tws_inflight) mbar_wait_bounded(w.bar_tws, w.ph_tws);
-  }
+  drain_copies(w, w.fail, w.fail && w.tws_inflight, mbar, NWG);
   fence_before_sync();
   __syncthreads();
   cluster_sync_all();

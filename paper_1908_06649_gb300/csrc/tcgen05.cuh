@@ -9,6 +9,8 @@
 namespace tcu {
 
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound per wait
+// bound of a failed kernel's wait for copies that may still be landing
+constexpr unsigned long long kDrainNs = 100000000ull;  // 0.1 s
 
 // ------------------------------------------------------------------ PTX glue
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -71,12 +73,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t parity) {
 // Bounded wait: true on success, false if the limit expired.  (A suspend-
 // time hint on try_wait measured slower here: waking costs more than the
 // polling it saves.)
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t parity,
+                                                  unsigned long long limit = kWaitNs) {
   if (mbar_try_wait(addr, parity)) return true;
   const unsigned long long t0 = global_ns();
   while (true) {
     if (mbar_try_wait(addr, parity)) return true;
-    if (global_ns() - t0 > kWaitNs) return false;
+    if (global_ns() - t0 > limit) return false;
   }
 }
 

@@ -1,10 +1,15 @@
-"""Order of the pass kernel's set-up, read from its source (CPU only).
+"""Order of the pass kernel's set-up and leaving, read from its source (CPU only).
 
 The next kernel of a stream may be placed on an SM as soon as every CTA of the
 running one has let it in.  Both want all of the SM's tensor memory, whose
 allocation has no time limit, so a CTA lets the next kernel in only when it
 holds its own: otherwise the next kernel could take the columns and wait for
-this kernel, while this kernel waits for the columns."""
+this kernel, while this kernel waits for the columns.
+
+A CTA whose wait ran out leaves with an error.  A bulk copy that has not landed
+by then would write into the shared memory of whoever gets the SM next, so it
+first waits until every mbarrier that copies complete on has nothing outstanding,
+whichever warp issued the copy and whichever wait failed."""
 import os
 import re
 
@@ -55,3 +60,25 @@ def test_every_thread_waits_for_the_kernels_before_it_touches_data():
     # neither a branch around the wait, nor an input copy or an early return before it
     assert head.count("{") - head.count("}") == 1
     assert "nx.issue(" not in head and "return;" not in head
+
+
+def test_a_failed_kernel_waits_for_every_copy_in_flight():
+    text = _source("group_kernel.cuh")
+    # the mbarriers that copies complete on: the staging's, the twiddles' and the tables'
+    bars = set(re.findall(r"mbar_expect_tx\(([^,]+),", text))
+    assert bars == {"w.bar_stg", "w.bar_tws", "smem_u32(tbar)"}
+    body = _body(text, "drain_copies")
+    assert "if (stg) drain_barrier(w.bar_stg);" in body
+    assert "if (tws) drain_barrier(w.bar_tws);" in body
+    assert "uint64_t *tbar = mbar + 3 * NWG + 1;" in _body(text, "kernel_setup_start")
+    assert "mbar_wait_bounded(smem_u32(mbar + 3 * nwg + 1), 0, kDrainNs)" in body
+    # whatever phase is incomplete: a thread's own phase bit has moved on when the
+    # wait for that copy ran out
+    assert "ph_" not in body + _body(text, "drain_barrier")
+    # the first copy counts before the warp that waits has issued one itself
+    assert "nx{P, &a.tm_in, item, nitems, item < nitems};" in _body(text, "dft_pass_kernel")
+    # the one-launch schedules: whatever their state says
+    for kernel in ("dft_fused_kernel", "dft_pair_kernel"):
+        assert re.search(r"(kernel_teardown\(tbase, w|drain_copies\(w), w\.fail, ",
+                         _body(text, kernel))
+    assert "drain_copies(" in _body(text, "kernel_teardown")
