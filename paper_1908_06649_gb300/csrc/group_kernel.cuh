@@ -1871,16 +1871,18 @@ __global__ void __launch_bounds__(
   // (gathered columns: every thread copies its own row, after the barrier)
   if (!G::GATHER && team == 0 && w.team_lead) nx.issue(w);
   const uint32_t tbase = kernel_setup_finish(tmem_slot);
-  // Only now, with this CTA's TMEM its own: a CTA of the next kernel that fits
-  // beside this one then waits in its allocation for this one to leave.  Let in
-  // earlier it could take the columns first and wait for this kernel, which would
-  // wait for them without a limit (today no two of these CTAs share an SM, by
-  // registers or by shared memory; nothing here rests on that).
-  launch_dependents();
   w.slot = tbase + (uint32_t)((threadIdx.x >> 7) * G::GCOLS);
   if (G::GATHER || (team != 0 && w.team_lead)) nx.issue(w);
   // the tables have landed (the same answer in every thread of the team)
   if (named_bar_or(w.bar_id, w.bar_count, !wait_tables(mbar, G::NWG))) w.fail = true;
+  // Only now, with this CTA's TMEM its own: a CTA of the next kernel that fits
+  // beside this one then waits in its allocation for this one to leave.  Let in
+  // earlier it could take the columns first and wait for this kernel, which would
+  // wait for them without a limit (today no two of these CTAs share an SM, by
+  // registers or by shared memory; nothing here rests on that).  Right after the
+  // allocation's barrier the compiler laid out the three-stage pass worse (16^3 x
+  // 16384 219 us against 210).
+  launch_dependents();
   while (item < nitems && !w.fail) {
     nx.next = item + istride;
     if constexpr (CONV != kNoConv)
