@@ -7,6 +7,14 @@
 
 namespace tcu {
 
+// The status of a launch.  A failure is read from the runtime, which would return
+// it again to the next launch that asks for the last error (the element-wise
+// kernels do), and so to a call whose kernels ran.
+inline cudaError_t launch_status(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // A pass kernel's launch: `sm` bytes of shared memory and, with `beside`, set up
 // beside the stream's previous kernel (programmatic serialization; the kernel
 // waits for it before it touches data), which takes 2-3 us off every launch:
@@ -15,7 +23,7 @@ inline cudaError_t launch_serial(void (*kernel)(const GArgs), long long grid, in
                                  size_t sm, bool beside, const GArgs &a, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return launch_status(e);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
@@ -27,7 +35,7 @@ inline cudaError_t launch_serial(void (*kernel)(const GArgs), long long grid, in
   attr[0].val.programmaticStreamSerializationAllowed = beside ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
+  return launch_status(cudaLaunchKernelEx(&cfg, kernel, a));
 }
 
 // Long radix-8 passes are launched after the kernel before them: CTAs that take
@@ -99,7 +107,7 @@ cudaError_t launch_fused_t(const GArgs &a, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(dft_fused_kernel<R, PREC, S1, S2>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return launch_status(e);
   dft_fused_kernel<R, PREC, S1, S2><<<(unsigned)num_sms, G1::THREADS, sm, st>>>(a);
   return cudaGetLastError();
 }
@@ -112,7 +120,7 @@ cudaError_t launch_pair_t(const GArgs &a, int clusters, cudaStream_t st) {
   const size_t sm = PL::BYTES;
   cudaError_t e = cudaFuncSetAttribute(dft_pair_kernel<R, PREC, S1, S2>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return launch_status(e);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
@@ -126,7 +134,7 @@ cudaError_t launch_pair_t(const GArgs &a, int clusters, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, dft_pair_kernel<R, PREC, S1, S2>, a);
+  return launch_status(cudaLaunchKernelEx(&cfg, dft_pair_kernel<R, PREC, S1, S2>, a));
 }
 
 #define TCU_PAIR_CASE(S1, S2)                                                       \
