@@ -998,12 +998,18 @@ __device__ __forceinline__ void gather_rows(const PRun &P, const WG &w, long lon
   const long long gi = (long long)tr * P.block - P.halo + q;
   const long long step = JS * P.side;  // a multiple of 8 floats
   const float *src = P.grid_in + gi * P.side + gj;
-  const uint32_t dst = smem_u32(w.stg + q * G::GG + ul);
+  const int i0 = q * G::GG + ul;  // staging [a][ul]
+  const uint32_t dst = smem_u32(w.stg + i0);
+  // index bounds of the checked build: of the staging, and of the grid from src
+  const long long values = P.side * P.side;
+  auto staged = [&](int j) { return in_range(w, i0 + j * (JS * G::GG), G::GPTS); };
   if (gi >= 0 && gi + (R - 1) * JS < P.side && gj >= 0 && gj + 1 < P.side &&
       ((uintptr_t)src & 7) == 0) {
     // inside the grid, on an 8-byte boundary in every row
 #pragma unroll
-    for (int j = 0; j < R; ++j, src += step) cp_async8(dst + j * (JS * G::GG * 8), src);
+    for (int j = 0; j < R; ++j, src += step)
+      if (staged(j) && in_range(w, src - P.grid_in, values - 1))
+        cp_async8(dst + j * (JS * G::GG * 8), src);
     return;
   }
   const bool in0 = gj >= 0 && gj < P.side, in1 = gj + 1 >= 0 && gj + 1 < P.side;
@@ -1011,8 +1017,11 @@ __device__ __forceinline__ void gather_rows(const PRun &P, const WG &w, long lon
   for (int j = 0; j < R; ++j, src += step) {
     const bool row = gi + j * JS >= 0 && gi + j * JS < P.side;
     const uint32_t at = dst + j * (JS * G::GG * 8);
-    cp_async4(at, row && in0 ? src : P.grid_in, row && in0);
-    cp_async4(at + 4, row && in1 ? src + 1 : P.grid_in, row && in1);
+    if (!staged(j)) continue;
+    if (!(row && in0) || in_range(w, src - P.grid_in, values))
+      cp_async4(at, row && in0 ? src : P.grid_in, row && in0);
+    if (!(row && in1) || in_range(w, src + 1 - P.grid_in, values))
+      cp_async4(at + 4, row && in1 ? src + 1 : P.grid_in, row && in1);
   }
 }
 
@@ -1036,18 +1045,20 @@ __device__ __forceinline__ void scatter_rows(const PRun &P, const WG &w, long lo
   const int rows = (int)min((long long)P.block, P.side - i0);
   const long long step = JS * P.side;
   float *dst = P.grid_out + (i0 + r0) * P.side + gj;
+  const long long values = P.side * P.side;  // index bound of the checked build
   if (in0 && in1 && ((uintptr_t)dst & 7) == 0) {  // on an 8-byte boundary in every row
 #pragma unroll
     for (int j = 0; j < R; ++j, dst += step)
-      if ((unsigned)(r0 + j * JS) < (unsigned)rows)
+      if ((unsigned)(r0 + j * JS) < (unsigned)rows &&
+          in_range(w, dst - P.grid_out, values - 1))
         __stcs(reinterpret_cast<float2 *>(dst), make_float2(d[2 * j], d[2 * j + 1]));
     return;
   }
 #pragma unroll
   for (int j = 0; j < R; ++j, dst += step)
     if ((unsigned)(r0 + j * JS) < (unsigned)rows) {
-      if (in0) __stcs(dst, d[2 * j]);
-      if (in1) __stcs(dst + 1, d[2 * j + 1]);
+      if (in0 && in_range(w, dst - P.grid_out, values)) __stcs(dst, d[2 * j]);
+      if (in1 && in_range(w, dst + 1 - P.grid_out, values)) __stcs(dst + 1, d[2 * j + 1]);
     }
 }
 
