@@ -1152,6 +1152,19 @@ __device__ __forceinline__ void last_stage_store(const PRun &P, long long item, 
   const long long toff = (klow << lgc) + uc, goff = ((long long)klow << G::LOG2VL) + vl;
   const long long gboff = (vh << G::LOG2L) + klow;
   const float2 one = make_float2(1.f, 0.f);
+  if constexpr (G::MODE_LAST == kRQF && S == 1) {
+    // One stage: a thread holds a whole transform, R contiguous outputs, and a warp's
+    // store touches 32 rows.  Such stores bound these passes (a row's sectors are
+    // written in parts), so they take 16 bytes each: n = 8 x 4194304 166 us with
+    // 8-byte stores (155 when a test of the spectrum spread them out), 88 so; n =
+    // 16 x 4194304 402 -> 263, 442 -> 265 in TF32; n = 32 x 2097152 395 -> 271.
+#pragma unroll
+    for (int j = 0; j < R; j += 2)
+      if (in_range(w, doff + j + 1, out_elems))
+        __stcs(reinterpret_cast<float4 *>(dst + j),
+               make_float4(d[2 * j], d[2 * j + 1], d[2 * j + 2], d[2 * j + 3]));
+    return;
+  }
   // The factors of a chunk of outputs (spectrum, twiddles) are loaded before
   // its stores: the stores are asm with a memory clobber, so a load written
   // after one of them would wait for it, a round trip per value.
