@@ -95,8 +95,9 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // strided pass 362 -> 335 us, 3-stage team pass 515 -> 451 us; 8^4 x 16384
 // last pass 175 -> 167 us); the 3-stage radix-8 passes on one-warpgroup items,
 // which work mostly in shared memory, keep five (8^3 x 100000: 168 us against
-// 174).  A
-// radix-16 first (strided) pass also stages its inter-pass twiddles
+// 174), and whole transforms of two stages run six (64 x 1000000: 155 us, 172
+// with eight, 164 with five; up to 64 x 100000, in L2, 16 us with six and eight,
+// 17 with five).  A radix-16 first (strided) pass also stages its inter-pass twiddles
 // in SMEM, which leaves room for four; a radix-16 last pass of several runs
 // four too (measured faster than five: 0.165 instead of 0.181 ms for the
 // second pass of n = 16^4 x 1024), and so does a column pass (256 x 256 x
@@ -108,12 +109,12 @@ __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 
 // per CTA at radix 32 (whole_k_nwg).  Convolution rows run four at radix 16
 // (registers: 256 x 256 x 500 303 -> 301 us, real tiles 170 -> 167).
 __host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
-  return R == 8    ? (S == 3 ? 5 : 8)
+  return R == 8    ? (S == 3 ? 5 : (S == 2 && ROLE == 0 ? 6 : 8))
          : R == 32 ? (S >= 2 ? 4 : 2)
                    : (ROLE != 0 && ROLE != 4 && ROLE != 7 ? 4 : 5);
 }
-__host__ __device__ constexpr int whole_k_nwg(int R, int ROLE, int S = 2) {
-  return R == 32 ? 2 : (R == 16 ? 4 : pass_nwg(R, ROLE, S));
+__host__ __device__ constexpr int whole_k_nwg(int R, int S = 2) {
+  return R == 32 ? 2 : (R == 16 ? 4 : (S == 3 ? 5 : 8));
 }
 // Warpgroups per CTA of a team pass: two teams of four at radix 8, two teams
 // of two at radix 16 (TMEM: 96 columns a slot; SMEM).
@@ -1838,11 +1839,11 @@ struct StaticNext {
 template <int R, int PREC, int S, int LO, int ROLE, int LP, int CONV = kNoConv, int TW = 1>
 __global__ void __launch_bounds__(
     Geo<R, S, LO, ROLE, LP,
-        TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>::THREADS,
+        TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>::THREADS,
     1) dft_pass_kernel(const __grid_constant__ GArgs a) {
   using G =
       Geo<R, S, LO, ROLE, LP,
-          TW == 1 ? (CONV ? whole_k_nwg(R, ROLE, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>;
+          TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>;
   static_assert(!CONV || ROLE == kSingle, "convolution rows are whole transforms");
   using SM = SmemLayout<R, G::NWG, G::TW_ENTRIES, CONV ? G::TW_ENTRIES : G::MIX_ENTRIES,
                         G::TW_SMEM, G::TWB, TW, G::KS>;
@@ -2113,10 +2114,10 @@ struct FusedNext {
 
 template <int R, int PREC, int S1, int S2>
 __global__ void __launch_bounds__(
-    Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R, kFirst)>::THREADS, 1)
+    Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R)>::THREADS, 1)
     dft_fused_kernel(const __grid_constant__ GArgs a) {
   static_assert(S1 >= 2 && S2 >= 2, "the fused schedule needs an SMEM barrier per item");
-  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R, kFirst)>;
+  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R)>;
   using G2 = Geo<R, S2, log2_radix(R) * S1, kSecond, 0, G1::NWG>;
   using SM = SmemLayout<R, G1::NWG, G1::TW_ENTRIES, G2::TW_ENTRIES, G1::TW_SMEM, G1::TWB>;
   constexpr int NWG = G1::NWG;
@@ -2523,7 +2524,7 @@ __device__ __forceinline__ void process_pair_item(const PRun &P, const float2 *t
 
 template <int R, int S1, int S2>
 struct PairLayout {
-  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R, kFirst)>;
+  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R)>;
   // no twiddle staging: pass-1 items read their inter-pass twiddles from
   // the L2-resident table while their last products run
   using SM = SmemLayout<R, G1::NWG, G1::TW_ENTRIES, Geo<R, S2, log2_radix(R) * S1, kSecond, 0,
@@ -2538,7 +2539,7 @@ struct PairLayout {
 
 template <int R, int PREC, int S1, int S2>
 __global__ void __launch_bounds__(
-    Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R, kFirst)>::THREADS, 1)
+    Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R)>::THREADS, 1)
     dft_pair_kernel(const __grid_constant__ GArgs a) {
   static_assert(S1 >= 2 && S2 >= 2, "the pair schedule needs an SMEM barrier per item");
   using PL = PairLayout<R, S1, S2>;

@@ -82,7 +82,7 @@ cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
 // The convolution row pass (forward rows, spectrum product, inverse rows).
 template <int R, int PREC, int S, int CONV>
 cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
-  using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, kSingle, S)>;
+  using G = Geo<R, S, 0, kSingle, 0, whole_k_nwg(R, S)>;
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::TW_ENTRIES, false, 0>::BYTES;
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
@@ -100,7 +100,7 @@ cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
 
 template <int R, int PREC, int S1, int S2>
 cudaError_t launch_fused_t(const GArgs &a, int num_sms, cudaStream_t st) {
-  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R, kFirst)>;
+  using G1 = Geo<R, S1, log2_radix(R) * S2, kFirst, 0, whole_k_nwg(R)>;
   using G2 = Geo<R, S2, log2_radix(R) * S1, kSecond, 0, G1::NWG>;
   const size_t sm =
       SmemLayout<R, G1::NWG, G1::TW_ENTRIES, G2::TW_ENTRIES, G1::TW_SMEM, G1::TWB>::BYTES;
