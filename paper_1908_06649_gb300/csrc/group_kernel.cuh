@@ -89,29 +89,33 @@ enum ConvMode { kNoConv = 0, kConv = 1, kRealConv = 2 };
 
 __host__ __device__ constexpr int log2_radix(int R) { return R == 8 ? 3 : (R == 16 ? 4 : 5); }
 // Warpgroups per CTA: TMEM holds 512 columns, a warpgroup's slot 3 Q of
-// them (Q = 2 R).  Radix 8 runs eight (slots of 48 columns, 64 registers a
-// thread): a row is only 8 values, so its threads are light and the pass is
-// bound by how many items are in flight (8^5 x 4096, five or four -> eight:
-// strided pass 362 -> 335 us, 3-stage team pass 515 -> 451 us; 8^4 x 16384
-// last pass 175 -> 167 us); the 3-stage radix-8 passes on one-warpgroup items,
-// which work mostly in shared memory, keep five (8^3 x 100000: 168 us against
-// 174), and whole transforms of two stages run six (64 x 1000000: 155 us, 172
-// with eight, 164 with five; up to 64 x 100000, in L2, 16 us with six and eight,
-// 17 with five).  A radix-16 first (strided) pass also stages its inter-pass twiddles
-// in SMEM, which leaves room for four; a radix-16 last pass of several runs
-// four too (measured faster than five: 0.165 instead of 0.181 ms for the
-// second pass of n = 16^4 x 1024), and so does a column pass (256 x 256 x
-// 1000 339 us against 363); whole mixed-radix transforms run five (512 x
-// 130000 204 us against 216).  A radix-32 pass of two stages runs
-// four warpgroups whose slots hold A for half of K (the products of a stage
-// in two K halves); one-stage radix-32 passes (already near the copy rate),
-// the convolution row pass and the fused schedule keep whole-K slots, two
-// per CTA at radix 32 (whole_k_nwg).  Convolution rows run four at radix 16
-// (registers: 256 x 256 x 500 303 -> 301 us, real tiles 170 -> 167).
-__host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2) {
-  return R == 8    ? (S == 3 ? 5 : (S == 2 && ROLE == 0 ? 6 : 8))
+// them (Q = 2 R).
+// Radix 8: eight (slots of 48 columns, 64 registers a thread).  A row is only 8
+// values, so threads are light and a pass is bound by how many items are in flight
+// (8^5 x 4096, five or four -> eight: strided pass 362 -> 335 us, 3-stage team pass
+// 515 -> 451 us; 8^4 x 16384 last pass 175 -> 167 us).  Three stages on
+// one-warpgroup items work mostly in shared memory and keep five (8^3 x 100000: 168
+// us against 174).  Whole transforms of two stages run six (64 x 1000000: 155 us,
+// 172 with eight, 164 with five; up to 64 x 100000, in L2, 16 us with six and
+// eight, 17 with five), as do the two-stage passes after a q-point pass (TF32, 960
+// x 34952: 186 us, 193 with eight).
+// Radix 16: four, five for whole transforms.  A strided pass also stages its
+// inter-pass twiddles in SMEM, which leaves room for four; a last pass of several
+// measured faster with four than with five (second pass of n = 16^4 x 1024 165 us
+// against 181), and so did a column pass (256 x 256 x 1000 339 us against 363).
+// Whole mixed-radix transforms run five (512 x 130000 204 us against 216), except
+// for one stage in TF32, whose sums from the definition spill at the registers of
+// five (176 x 190650 157 us against 165, 208 x 161319 180 against 181; in 3xTF32
+// the other way round, 182 against 174).
+// Radix 32: four for two stages, in slots that hold A for half of K (the products
+// of a stage in two K halves); one-stage passes, the convolution row pass and the
+// fused schedule keep whole-K slots, two per CTA (whole_k_nwg).
+// Convolution rows run four at radix 16 (registers: 256 x 256 x 500 303 -> 301 us,
+// real tiles 170 -> 167).
+__host__ __device__ constexpr int pass_nwg(int R, int ROLE, int S = 2, int PREC = 3) {
+  return R == 8    ? (S == 3 ? 5 : (S == 2 && (ROLE == 0 || ROLE == 4) ? 6 : 8))
          : R == 32 ? (S >= 2 ? 4 : 2)
-                   : (ROLE != 0 && ROLE != 4 && ROLE != 7 ? 4 : 5);
+                   : (ROLE == 0 || ROLE == 4 || (ROLE == 7 && (S > 1 || PREC != 1)) ? 5 : 4);
 }
 __host__ __device__ constexpr int whole_k_nwg(int R, int S = 2) {
   return R == 32 ? 2 : (R == 16 ? 4 : (S == 3 ? 5 : 8));
@@ -1839,11 +1843,12 @@ struct StaticNext {
 template <int R, int PREC, int S, int LO, int ROLE, int LP, int CONV = kNoConv, int TW = 1>
 __global__ void __launch_bounds__(
     Geo<R, S, LO, ROLE, LP,
-        TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>::THREADS,
+        TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S, PREC)) : team_nwg(R),
+        TW>::THREADS,
     1) dft_pass_kernel(const __grid_constant__ GArgs a) {
   using G =
       Geo<R, S, LO, ROLE, LP,
-          TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S)) : team_nwg(R), TW>;
+          TW == 1 ? (CONV ? whole_k_nwg(R, S) : pass_nwg(R, ROLE, S, PREC)) : team_nwg(R), TW>;
   static_assert(!CONV || ROLE == kSingle, "convolution rows are whole transforms");
   using SM = SmemLayout<R, G::NWG, G::TW_ENTRIES, CONV ? G::TW_ENTRIES : G::MIX_ENTRIES,
                         G::TW_SMEM, G::TWB, TW, G::KS>;

@@ -49,7 +49,7 @@ bool launch_beside(long long nitems, long long grid) {
 
 template <int R, int PREC, int S, int LO, int ROLE, int LP>
 cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
-  using G = Geo<R, S, LO, ROLE, LP>;
+  using G = Geo<R, S, LO, ROLE, LP, pass_nwg(R, ROLE, S, PREC)>;
   const size_t sm =
       SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, 1, G::KS>::BYTES;
   // one CTA per SM, each item on its own SM while there are fewer items
