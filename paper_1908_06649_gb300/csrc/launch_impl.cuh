@@ -38,13 +38,19 @@ inline cudaError_t launch_serial(void (*kernel)(const GArgs), long long grid, in
   return launch_status(cudaLaunchKernelEx(&cfg, kernel, a));
 }
 
-// Long radix-8 passes are launched after the kernel before them: CTAs that take
-// the SMs in the order they fall free left these passes 1-2 % slower (n = 32768 x
-// 4096: 780 us against 796, 4096 x 16384 342 against 346: 54 and more items a
-// team; 32768 x 1500, 39 items: 293 us against 289 beside).
-template <class G>
-bool launch_beside(long long nitems, long long grid) {
-  return G::LOG2R > 3 || nitems <= 45 * grid * G::NTEAM;
+// Long passes are launched after the kernel before them: CTAs that take the SMs in
+// the order they fall free no longer walk the arrays side by side, which costs more
+// than the 3 us a launch gained (n = 65536 x 512 168 us beside, 172 after; x 1024
+// 331, 332; x 2048 660, 655; 2^24 x 4 508, 511; x 8 1022, 1011; 2-D 1024^2 x 128
+// 790, 715).  The line lies between 67 and 84 million points; at radix 8 and with
+// one product in BF16, the lightest passes, between 49 and 64 (32768 x 1500, radix
+// 8: 289, 293; x 4096 796, 780; 2^20 x 45, radix 32 in BF16: 346, 346; x 61 464,
+// 459).  Whole transforms in one pass at radix 16 and 32 gain at any size (256 x
+// 400000 264, 268; 4096 x 32768 410, 413).
+template <class G, int PREC>
+bool launch_beside(bool whole, long long nitems) {
+  if (whole && G::LOG2R > 3) return true;
+  return nitems * G::GPTS <= (G::LOG2R == 3 || PREC == 4 ? 56 : 72) * 1000000ll;
 }
 
 template <int R, int PREC, int S, int LO, int ROLE, int LP>
@@ -56,8 +62,9 @@ cudaError_t launch_pass_t(const GArgs &a, int num_sms, cudaStream_t st) {
   // than SMs (latency), several per SM otherwise
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
+  const bool whole = ROLE == kSingle || ROLE == kSecondQF;
   return launch_serial(dft_pass_kernel<R, PREC, S, LO, ROLE, LP>, grid, G::THREADS, sm,
-                       launch_beside<G>(nitems, grid), a, st);
+                       launch_beside<G, PREC>(whole, nitems), a, st);
 }
 
 // A team pass: items of TW warpgroups (128 TW rows), team_nwg(R) warpgroups
@@ -68,8 +75,9 @@ cudaError_t launch_team_t(const GArgs &a, int num_sms, cudaStream_t st) {
   const size_t sm = SmemLayout<R, G::NWG, G::TW_ENTRIES, G::MIX_ENTRIES, G::TW_SMEM, G::TWB, TW>::BYTES;
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
-  return launch_serial(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>, grid,
-                       G::THREADS, sm, launch_beside<G>(nitems, grid), a, st);
+  const bool whole = ROLE == kSingle || ROLE == kSecondQF;
+  return launch_serial(dft_pass_kernel<R, PREC, S, LO, ROLE, LP, kNoConv, TW>, grid, G::THREADS,
+                       sm, launch_beside<G, PREC>(whole, nitems), a, st);
 }
 
 #define TCU_TEAM_CASE_L(S, LO, ROLE, LP, TW)                                             \
@@ -87,7 +95,7 @@ cudaError_t launch_rowconv_t(const GArgs &a, int num_sms, cudaStream_t st) {
   const long long nitems = pass_items<G>(a.p[0]);
   long long grid = nitems < num_sms ? nitems : num_sms;
   return launch_serial(dft_pass_kernel<R, PREC, S, 0, kSingle, 0, CONV>, grid, G::THREADS, sm,
-                       launch_beside<G>(nitems, grid), a, st);
+                       launch_beside<G, PREC>(false, nitems), a, st);
 }
 
 #define TCU_ROWCONV_CASE(S)                                                         \
