@@ -1877,10 +1877,12 @@ __global__ void __launch_bounds__(
   // two or more stages (1 %), half-K items (n = 1024 x 65536 173 -> 168 us), one
   // pass of three stages (16^3 x 16384 222 -> 215, 8^3 x 100000 147 -> 144),
   // convolution rows (radix-8 stencil of 4096^2 348 -> 335) and whole
-  // mixed-radix transforms on one warpgroup (192 x 200000 146 -> 142); not the
-  // last passes (three-stage radix-8 teams 435 -> 496) nor one-stage strided ones
-  if (((ROLE == kFirst || ROLE == kFirstQ) && S >= 2) || G::KS || CONV ||
-      (ROLE == kSingle && S == 3) || (G::SQ && TW == 1))
+  // mixed-radix transforms on one warpgroup (192 x 200000 146 -> 142).  Not the
+  // last passes (three-stage radix-8 teams 435 -> 496), one-stage strided ones,
+  // half-K items with one product in BF16 (32^4 x 61 464 -> 470) nor 16^3 in 3xBF16
+  // (x 32768 421 -> 427)
+  if (((ROLE == kFirst || ROLE == kFirstQ) && S >= 2 && !G::KS) || (G::KS && PREC != 4) ||
+      CONV || (ROLE == kSingle && S == 3 && !(R == 16 && PREC == 5)) || (G::SQ && TW == 1))
     w.copy_lead = (threadIdx.x >> 5) % (4 * TW) == 1;
 #ifdef TCU_DFT_CHECKED
   w.err = a.err;
