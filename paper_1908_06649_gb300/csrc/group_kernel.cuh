@@ -692,6 +692,9 @@ __device__ __forceinline__ float2 add_root(const RootsQ &r, float2 z, float2 x, 
 
 // y[k SY] = sum over i < Q of x[i SX] w_Q^{i k}, from the definition (DEF, or a
 // prime Q), else as Q1 x Q2 (Cooley-Tukey): 15 = 3 x 5 takes half the operations.
+// Sums over three of the partial sums take the roots of Q at once: a twiddle
+// product in between, rounded by itself, made 6 and 9 less exact than the
+// definition (error of n = 9 16 2.25e-7, 2.21e-7 from the definition, 2.19e-7 so).
 template <int Q0, int Q, int SX, int SY, bool DEF>
 __device__ __forceinline__ void dft_q(const RootsQ &r, const float2 *x, float2 *y) {
   constexpr int Q1 = DEF                    ? Q
@@ -716,12 +719,21 @@ __device__ __forceinline__ void dft_q(const RootsQ &r, const float2 *x, float2 *
       dft_q<Q0, Q1, Q2 * SX, Q2, DEF>(r, x + i2 * SX, t + i2);
 #pragma unroll
       for (int k1 = 1; k1 < Q1; ++k1)
-        if (i2 > 0)
+        if (Q2 != 3 && i2 > 0)
           t[k1 * Q2 + i2] =
               add_root<Q0, Q>(r, make_float2(0.f, 0.f), t[k1 * Q2 + i2], i2 * k1);
     }
 #pragma unroll
-    for (int k1 = 0; k1 < Q1; ++k1) dft_q<Q0, Q2, 1, Q1 * SY, DEF>(r, t + k1 * Q2, y + k1 * SY);
+    for (int k1 = 0; k1 < Q1; ++k1) {
+      if constexpr (Q2 == 3) {
+#pragma unroll
+        for (int k = k1; k < Q; k += Q1)
+          y[k * SY] = add_root<Q0, Q>(r, add_root<Q0, Q>(r, t[k1 * 3], t[k1 * 3 + 1], k),
+                                      t[k1 * 3 + 2], 2 * k % Q);
+      } else {
+        dft_q<Q0, Q2, 1, Q1 * SY, DEF>(r, t + k1 * Q2, y + k1 * SY);
+      }
+    }
   }
 }
 
