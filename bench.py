@@ -24,6 +24,7 @@ import argparse
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -164,6 +165,23 @@ class ClockSampler:
                     "samples": 0}
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": max(mx),
                 "reasons": sorted(reasons), "samples": len(sm)}
+
+
+def stencil_launches(precision, r, tile, steps):
+    """(real tiles, launches of a step, their names) of a stencil plan whose
+    tiles have one pass per axis.  3xTF32: real tiles, columns gathered, rows,
+    columns scattered, after the kernel's spectrum, directly (the library's line,
+    kClosedSteps, from its source) or from the weights: place, 2-D DFT (2), power,
+    inverse (2), kernel: place, 2-D DFT (2).  The other modes: the latter, and
+    complex tiles: gather, convolution (3), extract."""
+    src = open(os.path.join(ROOT, "paper_1908_06649_gb300", "csrc", "grid_plan.cu")).read()
+    closed = steps <= int(re.search(r"kClosedSteps = (\d+);", src).group(1))
+    if precision == 3 and tile <= {8: 512, 16: 256, 32: 1024}[r]:
+        rest = "gathered columns, convolution rows, scattered columns"
+        return ((True, 4, "kernel spectrum, " + rest) if closed else
+                (True, 12, "weights and kernel spectrum (9), " + rest))
+    return (False, 14, "weights and kernel spectrum (9), gather, columns, convolution "
+                       "rows, columns, extract")
 
 
 def kernel_sources_sha256():
@@ -457,12 +475,7 @@ def run_grid(args):
         tiles, Nt, B = pkg.stencil_tiles(side, k, r)
         points = tiles * Nt * Nt
         passes = 3
-        # 3xTF32 with tiles of one pass per axis: real tiles, columns gathered,
-        # rows, columns scattered; up to 20 steps the spectrum in one launch.
-        # Otherwise weights: place, 2-D DFT (2), power, inverse (2); kernel W':
-        # place, 2-D DFT (2); and complex tiles: gather, convolution (3), extract
-        real = args.precision == 3 and Nt <= {8: 512, 16: 256, 32: 1024}[r]
-        launches = (4 if k <= 20 else 12) if real else 14
+        real, launches, steps_text = stencil_launches(args.precision, r, Nt, k)
         unit = "Gupdates/s"
         metric = ("linear stencil grid-point updates/s (side^2 x steps), "
                   "%d^2 grid x %d steps, 1xGB300" % (side, k))
@@ -475,7 +488,8 @@ def run_grid(args):
                   "side": side, "steps": k, "sqrt_m": r, "tile": Nt, "block": B,
                   "l2": "grid %d MiB, but every step streams the %d MiB tile "
                         "batch through HBM three times, which evicts it; no "
-                        "flush" % (side * side * 4 >> 20, points * 8 >> 20)}
+                        "flush" % (side * side * 4 >> 20,
+                                   points * (4 if real else 8) >> 20)}
         value_of = lambda ms: side * side * k / (ms * 1e-3) / 1e9
         bytes_min = 8.0 * side * side
     for _ in range(max(3, args.warmup)):
@@ -509,8 +523,8 @@ def run_grid(args):
         step_bytes = (16.0 * points + 8.0 * S if real else
                       48.0 * points + 8.0 * points + 4.0 * S + 8.0 * S + 4.0 * S)
         achieved = step_bytes / (ms * 1e-3) / 1e9
-        kname = ("whole step (%d launches: kernel spectrum, gather, convolution "
-                 "rows, scatter), %.2f GB algorithmic" % (launches, step_bytes / 1e9))
+        kname = ("whole step (%d launches: %s), %.2f GB algorithmic"
+                 % (launches, steps_text, step_bytes / 1e9))
     else:
         achieved = 16.0 * points / (ms / passes * 1e-3) / 1e9
         kname = "average pass launch (%d pass launches per step)" % passes

@@ -232,7 +232,10 @@ int tcu_dft_exec_noalloc(int64_t n, int64_t batch, int32_t sqrt_m, int32_t preci
  * owned.  n1 and n2 are powers of sqrt_m with a 1-D plan each.  In the TF32
  * modes axes of at most one warpgroup pass (sqrt_m^2 for 16 and 32, 8^3 for 8)
  * with n1 * n2 >= 128 sqrt_m take two passes, columns then rows; the others
- * the rows' 1-D plan and up to three strided column passes.  Forward unscaled; inverse with the conjugate exponent and 1/(n1 n2).
+ * the rows' 1-D plan and up to three strided column passes (arrays smaller
+ * than one column item, n1 * n2 < 128 sqrt_m, and 4096 x 8 at sqrt_m = 8 in
+ * the single-product modes: transposes and a second 1-D plan).  Forward
+ * unscaled; inverse with the conjugate exponent and 1/(n1 n2).
  * tcu_dft2_plan allocates its tables and one batch-size scratch array and
  * returns NULL with tcu_dft_last_error() set on error (ERR_INVALID,
  * ERR_UNSUPPORTED, ERR_CUDA, ERR_OOM).  The exec calls are asynchronous on
@@ -245,8 +248,11 @@ int tcu_dft2_exec(tcu_dft2_plan_t p, const void *in, void *out, int dir, void *s
 /* out = IDFT2(DFT2(in) * spectrum) for every array of the batch: the
  * circular convolution of each array with the one n1 x n2 array whose 2-D
  * DFT is `spectrum` (device, n1*n2 complex64, e.g. from tcu_dft2_exec on a
- * batch-1 plan).  Three passes: columns; rows transformed, multiplied by
- * the spectrum and transformed back on chip; inverse columns. */
+ * batch-1 plan).  Two-pass plans take three passes: columns; rows
+ * transformed, multiplied by the spectrum and transformed back on chip;
+ * inverse columns.  The others transform rows and columns, multiply as the
+ * last column pass stores (or, between transposes, in a pass of its own) and
+ * transform columns and rows back. */
 int tcu_conv2_exec(tcu_dft2_plan_t p, const void *in, const void *spectrum, void *out,
                    void *stream);
 int tcu_dft2_check(tcu_dft2_plan_t p, void *stream);  /* as tcu_dft_check */
@@ -263,17 +269,21 @@ int tcu_dft2_destroy(tcu_dft2_plan_t p);                /* NULL: no-op, OK */
  *   inverse 2-D DFT, Nw the smallest power of sqrt_m >= 2k + 1.
  * tcu_stencil_exec: Lemma 1 -- output blocks of B x B points, B = N - 2k,
  *   N the smallest power of sqrt_m >= 3k (tcu_stencil_tiles): the (B + 2k) x
- *   (B + 2k) input
- *   window of every block (Lemma 1's 3k x 3k tile A'_{r,c} when B = k),
- *   zero-padded to N x N, convolved with the flipped, padded W as ONE batch,
- *   the B x B centres written to A_k (device, side^2 fp32; A_k == A
- *   allowed).  The result is the same for every B <= N - 2k; the largest
- *   makes the fewest tiles.
- * Needs N, Nw within one warpgroup pass (k <= 85 for sqrt_m 16, 170 for 8,
- * 341 for 32); else ERR_UNSUPPORTED.  Any side >= 1 (the last blocks of a
- * row or column are cut).  The plan allocates ceil(side/B)^2 N^2 complex64
- * of tiles plus tables; the calls are asynchronous on `stream` and allocate
- * nothing.  w3x3 is a host array. */
+ *   (B + 2k) input window of every block (Lemma 1's 3k x 3k tile A'_{r,c}
+ *   when B = k), zero-padded to N x N, convolved with the flipped, padded W
+ *   as ONE batch, the B x B centres written to A_k (device, side^2 fp32;
+ *   A_k == A allowed).  The result is the same for every B <= N - 2k; the
+ *   largest makes the fewest tiles.
+ * In 3xTF32 with N within one warpgroup pass (k <= 85 for sqrt_m 16, 170 for
+ * 8, 341 for 32) the tiles stay real, two columns packed as one complex one:
+ * three launches from the grid to the grid through ceil(side/B)^2 N^2/2
+ * complex64 of scratch, after the spectrum of W: up to 20 steps P(x,y)^k
+ * directly, in fp64 (one launch; W itself is not formed), beyond it by the
+ * transforms of Lemma 2.  Otherwise the windows become complex tiles, with
+ * ceil(side/B)^2 N^2 complex64 of tiles and as much scratch (N and Nw with a
+ * 2-D plan each, N^2 <= 2^26; else ERR_UNSUPPORTED).  Any side >= 1 (the last
+ * blocks of a row or column are cut).  The calls are asynchronous on `stream`
+ * and allocate nothing.  w3x3 is a host array. */
 typedef struct tcu_stencil_plan_s *tcu_stencil_plan_t;
 tcu_stencil_plan_t tcu_stencil_plan(int64_t side, int32_t steps, int32_t sqrt_m,
                                     int32_t precision);
@@ -283,9 +293,9 @@ int tcu_stencil_exec(tcu_stencil_plan_t p, const float *w3x3, const float *A, fl
 int tcu_stencil_check(tcu_stencil_plan_t p, void *stream);
 /* The tiling tcu_stencil_plan would choose, without a plan or a GPU: the
  * number of tiles ceil(side / B)^2 (0 if the arguments are unsupported), the
- * tile side N (the smallest power of sqrt_m with N >= 3k and N^2 >=
- * 128 sqrt_m, one warpgroup pass per axis) and the output block side
- * B = N - 2k, written to *tile and *block (either may be NULL). */
+ * tile side N (the smallest power of sqrt_m with N >= 3k and 128 sqrt_m <=
+ * N^2 <= 2^26) and the output block side B = N - 2k, written to *tile and
+ * *block (either may be NULL). */
 int64_t tcu_stencil_tiles(int64_t side, int32_t steps, int32_t sqrt_m, int64_t *tile,
                           int64_t *block);
 int tcu_stencil_destroy(tcu_stencil_plan_t p);

@@ -32,10 +32,9 @@ using namespace tcu::host;
 // passes of role kCols (the four-step split of the column length; the digit
 // reversal is in their output rows, so nothing is transposed).  HBM-bound: one
 // round trip per pass, two fewer than with a transpose each way (4096 x 4096 x 4
-// 929 -> 562 us, 256 x 256 x 1000 in BF16 788 -> 335, 65536 x 16 x 64
-// 1519 -> 766).  A
-// convolution multiplies by the spectrum as the last forward column pass
-// stores, then runs the inverse columns and rows.
+// 917 -> 534 us, 256 x 256 x 1000 in BF16 780 -> 321, 65536 x 16 x 64
+// 1504 -> 619).  A convolution multiplies by the spectrum as the last forward
+// column pass stores, then runs the inverse columns and rows.
 // Arrays smaller than one column item (n1 n2 < 128 r) transpose instead:
 // rows, transpose, the columns as rows, transpose back.
 struct tcu_dft2_plan_s {
@@ -59,9 +58,10 @@ struct tcu_dft2_plan_s {
 // untangles the rows 0 .. N / 2 of the column spectra (the others are their
 // conjugates), convolves them and packs them again; the inverse column pass
 // scatters the output blocks to the grid.  Half the transforms and a third of
-// the traffic of complex tiles (4096^2, 16 steps: 378 -> 153 us; 512^2 radix-8
-// tiles, 100 steps: 1053 -> 454).  The other modes keep complex
-// tiles: with single products every rounding of the operands would move.
+// the traffic of complex tiles (4096^2, 85 steps: 1666 -> 771 us; 512^2 radix-8
+// tiles, 100 steps: 1022 -> 400; with the spectrum below too, 16 steps 365 -> 128).
+// The other modes keep complex tiles: with single products every rounding of the
+// operands would move.
 struct tcu_stencil_plan_s {
   long long side, N, Nw, tiles;
   int B;  // output block side: N - 2k (Lemma 1's tiles are blocks of k)
@@ -78,11 +78,12 @@ struct tcu_stencil_plan_s {
 };
 
 // Steps up to which a real-tile plan evaluates the kernel's spectrum directly:
-// one launch instead of nine (a grid of 1000^2, 16 steps: 114 -> 31 us), and
-// more exact (error of the output 7.9e-6 -> 1.3e-6).  Beyond, the spectrum
-// comes from the transforms of Lemma 2, as tcu_stencil_weights' weights do:
-// their error grows with k (about 5e-7 k of the output), and results stay
-// within 2e-5 of theirs on either side of the line.
+// one launch instead of nine (a grid of 1000^2: 25 us with 20 steps, 50 with 21),
+// and more exact (error of the output with 16 steps 7.9e-6 -> 1.3e-6).  Neither
+// speed nor exactness sets the line: beyond it the spectrum comes, as before, from
+// the transforms of Lemma 2, as tcu_stencil_weights' weights do, whose error grows
+// with k (about 5e-7 k of the output), so that results stay within 2e-5 of what
+// those weights give on either side of the line.
 constexpr int kClosedSteps = 20;
 
 namespace {
@@ -563,7 +564,7 @@ long long grid_side(int r, long long need) {
 // N^2 >= 128 r (one warpgroup pass per axis); 0 if none.  Larger tiles give
 // larger output blocks (fewer tile points) but were measured slower per
 // point where they take three radix-8 stages per axis or radix-32 rows
-// (4096^2 x 16 steps: 512^2 tiles 1.31 ms against 0.856 ms for 64^2).
+// (4096^2 x 16 steps, complex tiles: 512^2 1.31 ms against 0.856 ms for 64^2).
 long long stencil_tile(int r, long long k, long long side) {
   (void)side;
   return grid_side(r, 3 * k);

@@ -195,8 +195,8 @@ struct Geo {
   static constexpr bool TW_OUT = ROLE == kFirst || ROLE == kFirstQ;
   // inter-pass twiddles staged by TMA per item (else read from the
   // L2-resident tables): measured faster for radix 16 and for the radix-8
-  // team items; the one-warpgroup radix-8 items run faster with five
-  // warpgroups and global reads, radix 32 has no SMEM to spare
+  // team items; the one-warpgroup radix-8 items run faster with more
+  // warpgroups (eight) and global reads, radix 32 has no SMEM to spare
   static constexpr bool TW_SMEM = TW_OUT && (R == 16 || (R == 8 && TW > 1));
   // w_M^{k v} with v = vh 2^VL + vl: table A [k][vl] and, for more than 256
   // columns, table B [vh][k] (two-level, so that no table exceeds L * 256)

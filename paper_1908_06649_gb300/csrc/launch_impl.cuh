@@ -18,7 +18,7 @@ inline cudaError_t launch_status(cudaError_t e) {
 // A pass kernel's launch: `sm` bytes of shared memory and, with `beside`, set up
 // beside the stream's previous kernel (programmatic serialization; the kernel
 // waits for it before it touches data), which takes 2-3 us off every launch:
-// n = 65536 x 64 30.6 -> 26.2 us a call, 4096^2 stencils 138 -> 131.
+// n = 65536 x 64 30.8 -> 26.0 us a call, 4096^2 stencils 136 -> 128.
 inline cudaError_t launch_serial(void (*kernel)(const GArgs), long long grid, int threads,
                                  size_t sm, bool beside, const GArgs &a, cudaStream_t st) {
   cudaError_t e =
